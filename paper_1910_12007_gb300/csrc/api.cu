@@ -157,7 +157,7 @@ extern "C" int swimmer_init(const swimmer_config *cfg, swimmer_handle **out) {
     CUDA_TRY(cudaDeviceGetAttribute(&h->regs_per_sm, cudaDevAttrMaxRegistersPerMultiprocessor, h->device));
     const int B = cfg->b_max;
     ALLOC(h->tab64, (size_t)B * TAB64_STRIDE);
-    ALLOC(h->k1_scratch, (size_t)B * K1_SCRATCH);
+    ALLOC(h->k1_scratch, (size_t)std::min(B, K1_SLICE) * K1_SCRATCH);
     ALLOC(h->tab32, (size_t)B * TAB32_STRIDE);
     ALLOC(h->pq, (size_t)B * cfg->n_max);
     ALLOC(h->sp, B);
@@ -350,7 +350,7 @@ extern "C" int swimmer_autotune(swimmer_handle *h, int steps, const double *thet
     for (int per = 1; per <= 17 && !rc; ++per, ++k) {
         const int B = (int)std::min<long long>((long long)per * h->num_sms, bmax);
         rc = launch_prepare(h, B, theta, nullptr, 0);
-        if (!rc) rc = launch_table_build(h, B, 1, 0);
+        if (!rc) rc = launch_table_build(h, B, prec == SWIMMER_FP64, 0);
         float best = 1e30f;
         int bestT = T0;
         for (int T = T0; T <= 1024 && !rc; T <<= 1) {

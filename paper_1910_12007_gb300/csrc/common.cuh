@@ -27,8 +27,9 @@ constexpr int TAB64_STRIDE = 2 * F64_PANELS_MAX * F64_NODES;
 // quadratic coefficients in G = 1 + f / F32_SUB, f in [0, 1) the local panel coordinate
 // (G is u's mantissa with the panel bits cleared)
 constexpr int TAB32_STRIDE = F32_PANELS_MAX + F32_PANELS_MAX / 2;
-constexpr int TAIL_MAX = 64;           // pieces of the integral of K0 phi s beyond the last node
-constexpr int K1_SCRATCH = 2 * NODES_MAX + TAIL_MAX;  // doubles of table-build scratch per sample
+constexpr int K1_ROWS = 8;             // values per node that the table build keeps in scratch
+constexpr int K1_SCRATCH = K1_ROWS * NODES_MAX + 16;  // doubles of table-build scratch per sample
+constexpr int K1_SLICE = 4096;         // samples whose tables are built at once (bounds the scratch)
 constexpr double R_MAX_OVER_L = 1.25;  // table reach in units of the flagellum length
 constexpr double STRETCH_MAX = 0.20;   // segment stretch beyond which a run counts as diverged
 constexpr int N_PTS_MAX = 1024;
@@ -105,7 +106,7 @@ struct swimmer_handle {
     int regs_per_sm;  // 32-bit registers per SM
     // per-sample workspace (b_max samples)
     double *tab64;          // [b_max][TAB64_STRIDE]
-    double *k1_scratch;     // [b_max][K1_SCRATCH] interval integrals of the table build
+    double *k1_scratch;     // [min(b_max, K1_SLICE)][K1_SCRATCH] node values of the table build
     float4 *tab32;          // [b_max][TAB32_STRIDE]
     float2 *pq;             // [b_max][n_max] FP32 kernel: preferred-curvature coefficients
     SampleParams *sp;       // [b_max]

@@ -13,20 +13,33 @@
 // where the bracketed differences are evaluated from their power series for x <= 2.
 // alpha = 0 is the regularized Stokeslet in closed form (Cortez 2001).
 //
-// Numerics (all FP64): Bessel I by power series (x <= 30) or the Hankel asymptotic
-// series; Bessel K by the A&S 9.6.11/9.6.13 series for x <= 2 and otherwise by the
-// trapezoid rule on K_nu(x) e^x = int_0^inf exp(-x (cosh t - 1)) cosh(nu t) dt, whose
-// error decays like exp(-2 pi d/h) for the strip half-width d = acos(1 - 1/x).  A1 and C
-// at the table nodes come from 16-point Gauss-Legendre integrals between consecutive
-// nodes, a warp prefix (A1) / suffix (C) sum and a geometric tail for C.
+// Numerics (all FP64).  The table's nodes lie at fixed u = 1 + sigma^2, sigma = r/delta, and so
+// do the Gauss-Legendre points of the integrals between consecutive nodes: sigma, ln sigma,
+// M0, the quadrature weights times phi s ds and the like are the same for every sample and are
+// made once per device (build_universal); a sample enters through beta = alpha delta alone,
+// x = beta sigma.  Each interval takes as many points as its distance from the integrands'
+// singularities (s = 0 and s = +-i delta) asks for 1e-16.  Bessel I: power series for x <= 8,
+// beyond that, and for K beyond x = 2, polynomials in 1/x fitted on the host at Chebyshev nodes
+// to sqrt(x) e^-x I and sqrt(x) e^x K (I from its power series and Hankel's expansion, K from
+// the trapezoid rule on K_nu(x) e^x = int_0^inf exp(-x (cosh t - 1)) cosh(nu t) dt); K for
+// x <= 2 from its ascending series (A&S 9.6.11/9.6.13).
 //
-// Output per sample: FP64 Chebyshev coefficients (8 panels per octave of
-// u = 1 + r^2/delta^2, degree 9) and, derived from them, FP32 quadratic coefficients in
-// the mantissa F in [1, 2) of u (64 panels per octave).
+// What bounds it: the FP64 pipe (two FMAs a clock and SM: a warp instruction takes 16 clocks).
+// Every integral by the trapezoid rule and a power series with FP64 tests, point by point, took
+// 20.6 ms for 1024 FP64 samples of N = 128 and 3.1 ms for a lone one; the fixed points and the
+// polynomials take 0.9 and 0.05 ms.  FP32 handles, whose arithmetic is fixed (below): 8.1 to
+// 2.3 ms for 1024 samples, 1.7 to 0.2 ms for 40, by taking both integrals of an interval at
+// the same points, the polynomial for K0 beyond x = 2, tests on the high words alone, and no
+// FP64 table beside the FP32 one.
+//
+// Output per sample: FP64 handles the FP64 table, FP32 handles quadratic coefficients in the
+// mantissa F in [1, 2) of u (64 panels per octave).
 #include <math.h>
 #include <stdio.h>
 
+#include <algorithm>
 #include <mutex>
+#include <vector>
 
 #include "common.cuh"
 
@@ -35,28 +48,143 @@ namespace {
 constexpr double PI = 3.14159265358979323846;
 constexpr double EGAMMA = 0.57721566490153286061;
 constexpr int GL_N = 16;
+// FP32 handles: the FP64 node values feed an FP32 table only, and ~1e-9 is enough: 6 nodes a panel
+constexpr int LITE_NODES = 6;
 __constant__ double c_gl_x[GL_N];   // 16-point Gauss-Legendre on [-1, 1]
 __constant__ double c_gl_w[GL_N];
-__constant__ double c_gl8_x[8];     // 8-point rule (FP32 handles: the table only feeds FP32)
-__constant__ double c_gl8_w[8];
-constexpr int NSER = 160;
-__constant__ double c_inv_k[NSER];          // 1/k (index 0 unused)
-__constant__ double c_inv_kk[2][NSER];      // 1/((k+1)(k+1+nu)) for nu = 0, 2
-__constant__ double c_cheb_t[F64_NODES];    // ascending Chebyshev nodes of the FP64 panels
+__constant__ double c_gl12_x[12];   // 12 points, for the tail
+__constant__ double c_gl12_w[12];
 __constant__ double c_dct[F64_NODES][F64_NODES];  // (2/n) cos(pi k (i + 1/2)/n), k = 0 halved
-// FP32 handles: the intermediate FP64 table needs only ~1e-9 (it feeds an FP32 table), so
-// its panels carry degree-5 series fitted at 6 nodes
-constexpr int LITE_NODES = 6;
-__constant__ double c_cheb_t6[LITE_NODES];
-__constant__ double c_dct6[LITE_NODES][LITE_NODES];
-__constant__ double c_node3[3];             // Chebyshev nodes for the FP32 quadratic fit
-__constant__ double c_dct3[3][3];
+// FP32 handles: 8 points, the 6 nodes' places and transform, the quadratic's 3 nodes
+__constant__ double c_gl8_x[8], c_gl8_w[8];
+__constant__ double c_cheb_t6[LITE_NODES], c_dct6[LITE_NODES][LITE_NODES];
+__constant__ double c_node3[3], c_dct3[3][3];
+constexpr int F32_SPLIT = F32_SUB / F64_SUB;  // FP32 panels per FP64 panel
+constexpr int NSER = 160;
+__constant__ double c_inv_k[NSER];      // 1/k (index 0 unused)
+__constant__ double c_inv_kk[2][NSER];  // 1/((k+1)(k+1+nu)) for nu = 0, 2
+constexpr int HARM = 64;
+__constant__ double c_harm[HARM];       // H_k, summed in order
+
+// Bessel coefficients (host-made): series in y = x^2/4, and polynomials in z = 1/x, each in its
+// range's variable t in [-1, 1]
+constexpr int SER = 25, SER_K = 13;
+__constant__ double c_i0[SER], c_i2[SER];       // 1/(k!)^2, 1/(k! (k+2)!)
+__constant__ double c_k0t[SER_K], c_t2[SER_K];  // H_k/(k!)^2, (H_k + H_{k+2})/(2 k! (k+2)!)
+constexpr int DEG_K = 16, DEG_I1 = 18, DEG_I2 = 12;
+constexpr double K_SPLIT = 6.0, I_SERIES = 8.0, I_SPLIT = 20.0;
+__constant__ double c_k0[2][DEG_K + 1], c_k1[2][DEG_K + 1];   // x in (2, 6], (6, inf)
+__constant__ double c_i0p[DEG_I1 + 1], c_i2p[DEG_I1 + 1];     // x in (8, 20]
+__constant__ double c_i0q[DEG_I2 + 1], c_i2q[DEG_I2 + 1];     // x in (20, inf)
+
+// FP64 handles: the sample-independent tables
+struct __align__(16) NodeRec {
+    double sig, lns, rsq, inv2, m0, pad;  // sigma, ln sigma, sigma^-1/2, sigma^-2, M0 (delta = 1)
+};
+struct __align__(16) QuadRec {
+    double sig, lns, rsq, w;  // a Gauss-Legendre point: w = weight * phi * sigma
+};
+constexpr int QUAD_MIN = 5;  // points of an interval at least
+constexpr int QUAD_CAP = 6 * NODES_MAX;
+__device__ NodeRec g_node[NODES_MAX];
+__device__ QuadRec g_quad[QUAD_CAP];
+__device__ int g_quad_at[NODES_MAX + 1];  // interval q: [at[q], at[q + 1])
+// beta times an interval's width beyond which its fixed points do not resolve e^(-beta s) (5
+// points: (beta w)^10 4e-13 relative); such intervals, far out where x > 40, are split anew
+constexpr double WIDTH_MAX = 0.7;
+
+template <int N>
+__device__ __forceinline__ double horner(const double *c, double t) {
+    double s = c[N - 1];
+#pragma unroll
+    for (int k = N - 2; k >= 0; --k) s = fma(s, t, c[k]);
+    return s;
+}
+
+// t in [-1, 1] of z = 1/x in [1/hi, 1/lo]
+__host__ __device__ constexpr double z_scale(double lo, double inv_hi) { return 2.0 / (1.0 / lo - inv_hi); }
+__host__ __device__ constexpr double z_shift(double lo, double inv_hi) { return -(1.0 / lo + inv_hi) / (1.0 / lo - inv_hi); }
+
+// polynomials of K_nu e^x sqrt(x) at z = 1/x, x > 2
+__device__ __forceinline__ double k_poly(const double (*c)[DEG_K + 1], bool far, double z) {
+    return far ? horner<DEG_K + 1>(c[1], fma(z, z_scale(K_SPLIT, 0.0), z_shift(K_SPLIT, 0.0)))
+               : horner<DEG_K + 1>(c[0], fma(z, z_scale(2.0, 1.0 / K_SPLIT), z_shift(2.0, 1.0 / K_SPLIT)));
+}
+
+// I_nu e^-x sqrt(x) at z = 1/x, x > 8
+__device__ __forceinline__ double i_poly(const double *p, const double *q, bool far, double z) {
+    return far ? horner<DEG_I2 + 1>(q, fma(z, z_scale(I_SPLIT, 0.0), z_shift(I_SPLIT, 0.0)))
+               : horner<DEG_I1 + 1>(p, fma(z, z_scale(I_SERIES, 1.0 / I_SPLIT), z_shift(I_SERIES, 1.0 / I_SPLIT)));
+}
+
+// K0(x), and I0(x) - 1 without cancellation when want_i.  lx = ln(x/2) + gamma and rs = x^(-1/2)
+// come with the point.
+__device__ __forceinline__ void bessel_k0_i0m1(double x, double lx, double rs, bool want_i, double &k0, double &i0m1) {
+    const double y = 0.25 * x * x;
+    if (x <= 2.0) {
+        // the series' lengths by size of y <= 1 (terms below 1e-18)
+        double im, tail;
+        if (y <= 0.0625) {
+            im = y * horner<7>(c_i0 + 1, y);
+            tail = y * horner<7>(c_k0t + 1, y);
+        } else {
+            im = y * horner<SER_K - 1>(c_i0 + 1, y);
+            tail = y * horner<SER_K - 1>(c_k0t + 1, y);
+        }
+        i0m1 = im;
+        k0 = fma(-lx, 1.0 + im, tail);  // K0 = -lx I0 + sum H_k y^k/(k!)^2
+        return;
+    }
+    const double z = rs * rs;
+    k0 = exp(-x) * rs * k_poly(c_k0, x > K_SPLIT, z);
+    if (want_i)
+        i0m1 = x <= I_SERIES ? y * horner<SER - 1>(c_i0 + 1, y)
+                             : exp(x) * rs * i_poly(c_i0p, c_i0q, x > I_SPLIT, z) - 1.0;
+}
 
 // ---------------------------------------------------------------------------------
-// Bessel functions
+// integrands and panel integrals
 // ---------------------------------------------------------------------------------
+// int_a^b f(s) ds (delta = 1), f = (I0(beta s) - 1) phi s and K0(beta s) phi s, split so that no
+// piece is wider than 0.5/beta or half the distance scale max(a, 1/4): the intervals whose
+// fixed points would not do
+__device__ __noinline__ void split_integral(double a, double b, double beta, double &ia, double &ic) {
+    const double w = b - a;
+    int n = (int)ceil(fmax(beta * w / 0.5, w / (0.5 * fmax(a, 0.25))));
+    n = n < 1 ? 1 : n > 4096 ? 4096 : n;
+    const double hw = 0.5 * w / n, lb = log(0.5 * beta) + EGAMMA;
+    ia = ic = 0.0;
+    for (int p = 0; p < n; ++p) {
+        const double c = a + (2 * p + 1) * hw;
+        for (int g = 0; g < GL_N; ++g) {
+            const double s = c + hw * c_gl_x[g], R2 = s * s + 1.0;
+            const double wt = hw * c_gl_w[g] * 3.0 * s / (2.0 * PI * R2 * R2 * sqrt(R2));
+            const double x = beta * s;
+            double k0, im = 0.0;
+            bessel_k0_i0m1(x, lb + log(s), rsqrt(x), true, k0, im);
+            ia = fma(wt, im, ia);
+            ic = fma(wt, k0, ic);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------------
+// FP32 handles.  Their tables are FP64 node values rounded to FP32 quadratics, and a run in
+// FP32 follows every rounding of them, so the arithmetic that a node value depends on to its last
+// bits (the recurrences, their order, the 8-point integrals) is fixed here, apart from that of the
+// FP64 handles above.  K0 inside the integral C enters a node value scaled by (delta/r)^3: beyond
+// x = 2 (in the tail: six units of x into it, and from the start where the weight is below 4e-6)
+// the polynomial above takes the place of the trapezoid rule, whose last bits no node value shows
+// there (bit-equal tables at 8000 samples of the sperm model, where the weight is largest).
+// ---------------------------------------------------------------------------------
+// term < 2^-e s for positive numbers from their high words alone: the series' tests, without
+// FP64 instructions (a term more or less lies below the sums' last bit)
+__device__ __forceinline__ bool below(double term, double s, int e) {
+    return __double2hiint(term) + (e << 20) < __double2hiint(s);
+}
+
 // I_nu(x), nu in {0, 2}: power series for x <= 30, Hankel asymptotic expansion beyond.
-__device__ double bessel_i(int nu, double x) {
+__device__ double series_i(int nu, double x) {
     if (x <= 30.0) {
         double y = 0.25 * x * x;
         double term = nu == 0 ? 1.0 : 0.5;  // 1/nu!
@@ -65,7 +193,7 @@ __device__ double bessel_i(int nu, double x) {
         for (int k = 0; k < NSER; ++k) {
             s += term;
             term *= y * inv[k];
-            if (term < 1e-18 * s) break;
+            if (below(term, s, 60)) break;
         }
         return s * (nu == 0 ? 1.0 : y);  // (x/2)^2 = y for nu = 2
     }
@@ -83,15 +211,45 @@ __device__ double bessel_i(int nu, double x) {
 }
 
 // I0(x) - 1 without cancellation
-__device__ double bessel_i0m1(double x) {
-    if (x > 1.0) return bessel_i(0, x) - 1.0;
+__device__ __forceinline__ double series_i0m1(double x) {
+    if (x > 1.0) return series_i(0, x) - 1.0;
     double y = 0.25 * x * x, term = y, s = 0.0;
     for (int k = 1; k < 60; ++k) {
         s += term;
         term *= y * c_inv_kk[0][k];  // 1/((k+1)^2)
-        if (term < 1e-18 * s) break;
+        if (below(term, s, 60)) break;
     }
     return s;
+}
+
+// K0(x) for x <= 2 = -(ln(x/2) + gamma) I0(x) + sum_{k>=1} H_k y^k/(k!)^2, y = x^2/4 (one pass)
+__device__ __forceinline__ double series_k0(double x) {
+    double y = 0.25 * x * x, term = 1.0, i0 = 1.0, tail = 0.0;
+    for (int k = 1; k < 60; ++k) {
+        term *= y * c_inv_kk[0][k - 1];
+        i0 += term;
+        tail += c_harm[k] * term;
+        if (below(term, i0, 63)) break;
+    }
+    return -(log(0.5 * x) + EGAMMA) * i0 + tail;
+}
+
+// K0(x) for x > 2 by the trapezoid rule on K0(x) e^x = int_0^inf exp(-x (cosh t - 1)) dt
+__device__ __noinline__ double trapezoid_k0(double x) {
+    double d = acos(1.0 - 1.0 / x);
+    double h = d / 6.5;
+    double s0 = 0.5;
+    const double eh = exp(h), emh = 1.0 / eh;
+    double ep = 1.0, em = 1.0;  // e^{m h}, e^{-m h}
+    for (int m = 1; m < 4000; ++m) {
+        ep *= eh;
+        em *= emh;
+        double c = 0.5 * (ep + em);  // cosh(m h)
+        double e = exp(-x * (c - 1.0));
+        s0 += e;
+        if (below(e, s0, 63)) break;
+    }
+    return h * s0 * exp(-x);
 }
 
 struct BesselSet {
@@ -99,7 +257,7 @@ struct BesselSet {
 };
 
 // K0(x) e^x and K1(x) e^x for x > 2 by the trapezoid rule on the integral representation
-__device__ void bessel_k01_scaled(double x, double *k0e, double *k1e) {
+__device__ void trapezoid_k01(double x, double *k0e, double *k1e) {
     double d = acos(1.0 - 1.0 / x);
     double h = d / 6.5;
     double s0 = 0.5, s1 = 0.5;
@@ -112,7 +270,7 @@ __device__ void bessel_k01_scaled(double x, double *k0e, double *k1e) {
         double e = exp(-x * (c - 1.0));
         s0 += e;
         s1 += e * c;
-        if (e < 1e-19 * s0) break;
+        if (below(e, s0, 63)) break;
     }
     *k0e = h * s0;
     *k1e = h * s1;
@@ -120,18 +278,17 @@ __device__ void bessel_k01_scaled(double x, double *k0e, double *k1e) {
 
 __device__ BesselSet bessel_set(double x) {
     BesselSet b;
-    b.i0 = bessel_i(0, x);
-    b.i2 = bessel_i(2, x);
+    b.i0 = series_i(0, x);
+    b.i2 = series_i(2, x);
     if (x <= 2.0) {
         double y = 0.25 * x * x;
         double lx = log(0.5 * x) + EGAMMA;
         // K0 = -lx I0 + sum_{k>=1} H_k y^k/(k!)^2
-        double term = 1.0, hk = 0.0, tail = 0.0;
+        double term = 1.0, tail = 0.0;
         for (int k = 1; k < 60; ++k) {
             term *= y * c_inv_kk[0][k - 1];  // 1/k^2
-            hk += c_inv_k[k];
-            tail += hk * term;
-            if (term < 1e-19) break;
+            tail += c_harm[k] * term;
+            if (below(term, 1.0, 63)) break;
         }
         b.k0 = -lx * b.i0 + tail;
         // 2/x^2 - K2 = 1/2 + y sum_k [lx - (H_k + H_{k+2})/2] y^k/(k!(k+2)!)
@@ -143,14 +300,14 @@ __device__ BesselSet bessel_set(double x) {
             term *= y * c_inv_kk[1][k];  // 1/((k+1)(k+3))
             hk0 += c_inv_k[k + 1];
             hk2 += c_inv_k[k + 3];
-            if (term < 1e-20) break;
+            if (below(term, 1.0, 66)) break;
         }
         b.t2k2 = 0.5 + y * s;
         b.k2 = 2.0 / (x * x) - b.t2k2;
         b.ix2w = 0.5 * b.t2k2 - 0.5 * b.k0;
     } else {
         double k0e, k1e;
-        bessel_k01_scaled(x, &k0e, &k1e);
+        trapezoid_k01(x, &k0e, &k1e);
         double ex = exp(-x);
         b.k0 = k0e * ex;
         double k1 = k1e * ex;
@@ -161,27 +318,6 @@ __device__ BesselSet bessel_set(double x) {
     return b;
 }
 
-__device__ double bessel_k0(double x) {
-    if (x <= 2.0) {
-        // K0 = -(ln(x/2) + gamma) I0 + sum_{k>=1} H_k y^k/(k!)^2, y = x^2/4 (one pass)
-        double y = 0.25 * x * x, term = 1.0, i0 = 1.0, hk = 0.0, tail = 0.0;
-        for (int k = 1; k < 60; ++k) {
-            term *= y * c_inv_kk[0][k - 1];
-            hk += c_inv_k[k];
-            i0 += term;
-            tail += hk * term;
-            if (term < 1e-19 * i0) break;
-        }
-        return -(log(0.5 * x) + EGAMMA) * i0 + tail;
-    }
-    double k0e, k1e;
-    bessel_k01_scaled(x, &k0e, &k1e);
-    return k0e * exp(-x);
-}
-
-// ---------------------------------------------------------------------------------
-// integrands and panel integrals
-// ---------------------------------------------------------------------------------
 __device__ __forceinline__ double blob(double s, double delta) {
     double R2 = s * s + delta * delta;
     return 3.0 * delta * delta * delta / (2.0 * PI * R2 * R2 * sqrt(R2));
@@ -192,35 +328,43 @@ __device__ double m0_closed(double r, double delta) {
     return (r * r / (R + delta)) * (R * R + R * delta + delta * delta) / (R * R * R) / (2.0 * PI);
 }
 
-// int_a^b f(s) ds with f = (I0(alpha s)-1) phi s (which = 0) or K0(alpha s) phi s (which = 1),
-// split so that no piece is wider than 0.5/alpha or half the distance scale max(a, delta/4)
-__device__ double panel_integral(int which, double a, double b, double alpha, double delta, bool gl8) {
-    if (b <= a) return 0.0;
+__device__ __forceinline__ double node6_u(int m) {
+    // node m -> (octave, panel, ascending Chebyshev index)
+    int panel = m / LITE_NODES, ii = m % LITE_NODES;
+    int e = panel >> F64_SUB_LOG2, j = panel & (F64_SUB - 1);
+    double f = 0.5 * (c_cheb_t6[ii] + 1.0);
+    return ldexp(1.0 + (j + f) / F64_SUB, e);
+}
+
+// int_a^b of (I0(alpha s) - 1) phi s and of K0(alpha s) phi s, 8 points a piece, split so that no
+// piece is wider than 0.5/alpha or half the distance scale max(a, delta/4)
+__device__ void panel_integrals8(double a, double b, double alpha, double delta, bool want_k, double &ia, double &ic) {
     double w = b - a;
     int n = (int)ceil(fmax(alpha * w / 0.5, w / (0.5 * fmax(a, 0.25 * delta))));
     if (n < 1) n = 1;
     if (n > 4096) n = 4096;
-    const int ng = gl8 ? 8 : GL_N;
-    const double *gx = gl8 ? c_gl8_x : c_gl_x, *gw = gl8 ? c_gl8_w : c_gl_w;
-    double hw = 0.5 * w / n, tot = 0.0;
+    double hw = 0.5 * w / n, ta = 0.0, tc = 0.0;
     for (int p = 0; p < n; ++p) {
-        double c = a + (2 * p + 1) * hw, acc = 0.0;
-        for (int g = 0; g < ng; ++g) {
-            double s = c + hw * gx[g];
-            double f = (which == 0 ? bessel_i0m1(alpha * s) : bessel_k0(alpha * s)) * blob(s, delta) * s;
-            acc += gw[g] * f;
+        double c = a + (2 * p + 1) * hw, aa = 0.0, ac = 0.0;
+        for (int g = 0; g < 8; ++g) {
+            double s = c + hw * c_gl8_x[g], x = alpha * s, bl = blob(s, delta);
+            double f = series_i0m1(x) * bl * s;
+            aa += c_gl8_w[g] * f;
+            if (want_k) {
+                double k0, im;
+                if (x <= 2.0)
+                    k0 = series_k0(x);
+                else
+                    bessel_k0_i0m1(x, 0.0, rsqrt(x), false, k0, im);
+                f = k0 * bl * s;
+                ac += c_gl8_w[g] * f;
+            }
         }
-        tot += acc * hw;
+        ta += aa * hw;
+        tc += ac * hw;
     }
-    return tot;
-}
-
-__device__ __forceinline__ double node_u(int m, int np) {
-    // node m -> (octave, panel, ascending Chebyshev index); np nodes per panel
-    int panel = m / np, ii = m % np;
-    int e = panel >> F64_SUB_LOG2, j = panel & (F64_SUB - 1);
-    double f = 0.5 * ((np == F64_NODES ? c_cheb_t[ii] : c_cheb_t6[ii]) + 1.0);
-    return ldexp(1.0 + (j + f) / F64_SUB, e);
+    ia = ta;
+    ic = tc;
 }
 
 __device__ void stokes_g(double r, double delta, double *g1, double *g2) {
@@ -300,106 +444,264 @@ __global__ void __launch_bounds__(SORT_THREADS) order_kernel(int B, const Sample
 }
 
 // ---------------------------------------------------------------------------------
-// K1a: interval integrals, one thread per node interval or tail piece (all samples)
+// K1a: one thread per node: the integrals over the interval that ends at the node and the
+// Bessel factors at the node, for all samples; the last row of CTAs takes the integral of
+// K0 phi s beyond the last node
 // ---------------------------------------------------------------------------------
 constexpr int K1_THREADS = 256;
 constexpr int K1A_THREADS = 128;
+// tail pieces beyond sigma_last: each sqrt(2) - 1 of its start wide, at most 4/beta, until 60/beta
+// beyond or s^-3 has fallen by 1e-18; 12 points a piece
+constexpr int TAIL_PIECES = 60, TAIL_POINTS = 12;
+// FP32 handles: at most 64 pieces of up to 5 parts (a piece is at most 2/alpha wide, a part
+// 0.5/alpha; 5 by rounding), 8 points a part.  The last of 64 pieces runs to the end whatever
+// its width: with as many its share is below 1e-18 of the first's.
+constexpr int TAIL8_MAX = 64, TAIL8_SUB = 5, TAIL8_POINTS = TAIL8_MAX * TAIL8_SUB * 8;
 
 __device__ __forceinline__ int node_count(const SampleParams &p, int NP, int max_oct) {
     return min(p.n_oct, max_oct) * F64_SUB * NP;
 }
 
-// tail piece k beyond r_last: widths double from the blob scale up to 2/alpha, then stay;
-// the last piece ends at s_end.  Returns false when piece k does not exist.
-__device__ bool tail_piece(int k, double r_last, double s_end, double alpha, double delta, double *lo, double *hi) {
-    double s = r_last;
-    for (int i = 0; i < TAIL_MAX; ++i) {
-        if (s >= s_end) return false;
-        double w = fmin(fmax(s, 0.25 * delta), 2.0 / alpha);
-        double e = (i == TAIL_MAX - 1) ? s_end : fmin(s + w, s_end);
-        if (i == k) {
-            *lo = s;
-            *hi = e;
-            return true;
-        }
-        s = e;
-    }
-    return false;
-}
+// scratch row of a sample: K1_ROWS values per node, then the tail
+enum { K1_IA, K1_IC, K1_E1, K1_WA, K1_WC, K1_E2, K1_VA, K1_VC };
+enum { K1_I0 = 2, K1_I2, K1_K0, K1_K2, K1_T2K2, K1_IX2W };  // FP32 handles
 
 __global__ void __launch_bounds__(K1A_THREADS)
-table_integrals_kernel(int B, const SampleParams *__restrict__ sp, double *__restrict__ scratch, int gl8,
-                       int max_oct) {
-    const int b = blockIdx.x;
-    const SampleParams p = sp[b];
+table_nodes_kernel(const SampleParams *__restrict__ sp, double *__restrict__ scratch, int lite, int max_oct) {
+    __shared__ double s_edge[TAIL8_MAX + 1], s_red[K1A_THREADS / 32];
+    __shared__ int s_pieces, s_at[TAIL8_MAX + 1];
+    static_assert(TAIL_PIECES <= TAIL8_MAX && TAIL8_MAX <= K1A_THREADS, "tail pieces");
+    const SampleParams p = sp[blockIdx.x];
     if (p.status != SWIMMER_OK || !(p.alpha > 0.0)) return;
-    const int NP = gl8 ? LITE_NODES : F64_NODES;
+    const int NP = lite ? LITE_NODES : F64_NODES;
     const int M = node_count(p, NP, max_oct);
-    const int q = blockIdx.y * blockDim.x + threadIdx.x;
-    const double alpha = p.alpha, delta = p.delta;
-    double *IA = scratch + (size_t)b * K1_SCRATCH, *IC = IA + NODES_MAX, *IT = IC + NODES_MAX;
-    if (q < M) {
-        double r = delta * sqrt(node_u(q, NP) - 1.0);
-        double rprev = q ? delta * sqrt(node_u(q - 1, NP) - 1.0) : 0.0;
-        IA[q] = panel_integral(0, rprev, r, alpha, delta, gl8);
-        IC[q] = q + 1 < M ? panel_integral(1, r, delta * sqrt(node_u(q + 1, NP) - 1.0), alpha, delta, gl8) : 0.0;
-    } else if (q < M + TAIL_MAX) {
-        const int k = q - M;
-        double r_last = delta * sqrt(node_u(M - 1, NP) - 1.0);
-        double s_end = fmin(r_last + 60.0 / alpha, 1e6 * delta);
-        double lo, hi;
-        IT[k] = tail_piece(k, r_last, s_end, alpha, delta, &lo, &hi) ? panel_integral(1, lo, hi, alpha, delta, gl8) : 0.0;
+    const double beta = p.alpha * p.delta;
+    double *out = scratch + (size_t)blockIdx.x * K1_SCRATCH;
+    if (lite && blockIdx.y == gridDim.y - 1) {
+        // the tail: pieces whose widths double from the last node up to 2/alpha, then stay; a
+        // thread per point, then a thread per piece sums its points in order
+        __shared__ double s_f[TAIL8_POINTS];
+        if (threadIdx.x == 0) {
+            const double r_last = p.delta * sqrt(node6_u(M - 1) - 1.0);
+            const double end = fmin(r_last + 60.0 / p.alpha, 1e6 * p.delta);
+            double s = r_last;
+            int k = 0, at = 0;
+            while (k < TAIL8_MAX && s < end) {
+                const double w = fmin(fmax(s, 0.25 * p.delta), 2.0 / p.alpha);
+                const double e = (k == TAIL8_MAX - 1) ? end : fmin(s + w, end);
+                s_edge[k] = s;
+                const double we = e - s;
+                int n = (int)ceil(fmax(p.alpha * we / 0.5, we / (0.5 * fmax(s, 0.25 * p.delta))));
+                s_at[k] = at;
+                at += n < 1 ? 1 : n > TAIL8_SUB ? TAIL8_SUB : n;
+                s = e;
+                s_edge[++k] = s;
+            }
+            s_at[k] = at;
+            s_pieces = k;
+        }
+        __syncthreads();
+        const int K = s_pieces;
+        const double dr = p.delta / s_edge[0];
+        const double x_exact = dr * dr * dr > 4e-6 ? p.alpha * s_edge[0] + 6.0 : 2.0;
+        for (int i = threadIdx.x; i < 8 * s_at[K]; i += K1A_THREADS) {
+            int k = 0;
+            while (s_at[k + 1] <= i / 8) ++k;
+            const int n = s_at[k + 1] - s_at[k], q = i / 8 - s_at[k];
+            const double hw = 0.5 * (s_edge[k + 1] - s_edge[k]) / n, c = s_edge[k] + (2 * q + 1) * hw;
+            const double s = c + hw * c_gl8_x[i % 8], x = p.alpha * s;
+            double k0, im;
+            if (x <= 2.0)
+                k0 = series_k0(x);
+            else if (x <= x_exact)
+                k0 = trapezoid_k0(x);
+            else
+                bessel_k0_i0m1(x, 0.0, rsqrt(x), false, k0, im);
+            s_f[i] = k0 * blob(s, p.delta) * s;
+        }
+        __syncthreads();
+        double tot = 0.0;
+        if (threadIdx.x < K) {
+            const int k = threadIdx.x, n = s_at[k + 1] - s_at[k];
+            const double hw = 0.5 * (s_edge[k + 1] - s_edge[k]) / n;
+            for (int q = 0; q < n; ++q) {
+                double acc = 0.0;
+                for (int g = 0; g < 8; ++g) acc += c_gl8_w[g] * s_f[8 * (s_at[k] + q) + g];
+                tot += acc * hw;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < K) s_f[threadIdx.x] = tot;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int k = K - 1; k >= 0; --k) t += s_f[k];  // far (small) pieces first
+            out[K1_ROWS * (size_t)NODES_MAX] = t;
+        }
+        return;
     }
+    if (blockIdx.y == gridDim.y - 1) {  // the tail
+        const double s0 = g_node[M - 1].sig;
+        if (threadIdx.x == 0) {
+            double s = s0;
+            const double wmax = 4.0 / beta, end = s0 + 60.0 / beta, last = fmin(1e6, 1e6 * s0);
+            int k = 0;
+            s_edge[0] = s;
+            while (k < TAIL_PIECES && s < end && s < last) {
+                s = fmin(s + fmin(0.41421356237309515 * s, wmax), end);
+                s_edge[++k] = s;
+            }
+            s_pieces = k;
+        }
+        __syncthreads();
+        const double lb = log(0.5 * beta) + EGAMMA;
+        double sum = 0.0;
+        for (int i = threadIdx.x; i < s_pieces * TAIL_POINTS; i += K1A_THREADS) {
+            const int k = i / TAIL_POINTS, g = i % TAIL_POINTS;
+            const double a = s_edge[k], hw = 0.5 * (s_edge[k + 1] - a);
+            const double s = a + hw + hw * c_gl12_x[g], q = rsqrt(fma(s, s, 1.0)), q2 = q * q, x = beta * s;
+            double k0, im;
+            bessel_k0_i0m1(x, lb + log(s), rsqrt(x), false, k0, im);
+            sum = fma(hw * c_gl12_w[g] * (3.0 / (2.0 * PI)) * s * q2 * q2 * q, k0, sum);
+        }
+        for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = sum;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int k = 0; k < K1A_THREADS / 32; ++k) t += s_red[k];
+            out[K1_ROWS * (size_t)NODES_MAX] = t;
+        }
+        return;
+    }
+    const int q = blockIdx.y * K1A_THREADS + threadIdx.x;
+    if (q >= M) return;
+    // ---- the interval [sigma_{q-1}, sigma_q] (from 0 for the first node, where only A1's counts)
+    double ia = 0.0, ic = 0.0;
+    if (lite) {
+        const double r = p.delta * sqrt(node6_u(q) - 1.0), rprev = q ? p.delta * sqrt(node6_u(q - 1) - 1.0) : 0.0;
+        panel_integrals8(rprev, r, p.alpha, p.delta, q > 0, ia, ic);
+        const BesselSet bs = bessel_set(p.alpha * r);
+        out[K1_IA * (size_t)NODES_MAX + q] = ia;
+        out[K1_IC * (size_t)NODES_MAX + q] = ic;
+        out[K1_I0 * (size_t)NODES_MAX + q] = bs.i0;
+        out[K1_I2 * (size_t)NODES_MAX + q] = bs.i2;
+        out[K1_K0 * (size_t)NODES_MAX + q] = bs.k0;
+        out[K1_K2 * (size_t)NODES_MAX + q] = bs.k2;
+        out[K1_T2K2 * (size_t)NODES_MAX + q] = bs.t2k2;
+        out[K1_IX2W * (size_t)NODES_MAX + q] = bs.ix2w;
+        return;
+    }
+    const double lb = log(0.5 * beta) + EGAMMA, rsb = rsqrt(beta);
+    const NodeRec nd = g_node[q];
+    const double sprev = q ? g_node[q - 1].sig : 0.0;
+    if (beta * (nd.sig - sprev) > WIDTH_MAX) {
+        split_integral(sprev, nd.sig, beta, ia, ic);
+    } else {
+        const int e = g_quad_at[q + 1];
+        for (int i = g_quad_at[q]; i < e; ++i) {
+            const QuadRec c = g_quad[i];
+            double k0, im = 0.0;
+            bessel_k0_i0m1(beta * c.sig, lb + c.lns, rsb * c.rsq, true, k0, im);
+            ia = fma(c.w, im, ia);
+            ic = fma(c.w, k0, ic);
+        }
+    }
+    out[K1_IA * (size_t)NODES_MAX + q] = ia;
+    out[K1_IC * (size_t)NODES_MAX + q] = ic;
+    // ---- the node: g1 = E1 - WA A1 - WC C, delta^2 g2 = E2 - VA A1 - VC C
+    const double x = beta * nd.sig, rs = rsb * nd.rsq, z = rs * rs;
+    double i0, i2, k0, k2, t2k2, ix2w;  // t2k2 = 2/x^2 - K2, ix2w = 1/x^2 - (K0 + K2)/2
+    const double y = 0.25 * x * x, lx = lb + nd.lns;
+    if (x <= I_SERIES) {
+        if (x <= 2.0) {
+            i0 = horner<SER_K>(c_i0, y);
+            i2 = horner<SER_K>(c_i2, y);
+        } else {
+            i0 = horner<SER>(c_i0, y);
+            i2 = horner<SER>(c_i2, y);
+        }
+    } else {
+        const double ex = exp(x) * rs;
+        i0 = ex * i_poly(c_i0p, c_i0q, x > I_SPLIT, z);
+        i2 = ex * i_poly(c_i2p, c_i2q, x > I_SPLIT, z);
+    }
+    if (x <= 2.0) {
+        k0 = fma(-lx, i0, y * horner<SER_K - 1>(c_k0t + 1, y));
+        // 2/x^2 - K2 = 1/2 + y sum_k [lx - (H_k + H_{k+2})/2] y^k/(k! (k+2)!)
+        t2k2 = fma(y, fma(lx, i2, -horner<SER_K>(c_t2, y)), 0.5);
+        k2 = 0.5 / y - t2k2;
+        ix2w = 0.5 * (t2k2 - k0);
+        i2 *= y;
+    } else {
+        const double ex = exp(-x) * rs;
+        const bool far = x > K_SPLIT;
+        k0 = ex * k_poly(c_k0, far, z);
+        k2 = fma(2.0 * z, ex * k_poly(c_k1, far, z), k0);
+        t2k2 = fma(2.0 * z, z, -k2);
+        ix2w = fma(z, z, -0.5 * (k0 + k2));
+        if (x <= I_SERIES) i2 *= y;
+    }
+    out[K1_E1 * (size_t)NODES_MAX + q] = ix2w * nd.m0;
+    out[K1_WA * (size_t)NODES_MAX + q] = 0.5 * (k0 + k2);
+    out[K1_WC * (size_t)NODES_MAX + q] = 0.5 * (i0 + i2);
+    out[K1_E2 * (size_t)NODES_MAX + q] = t2k2 * nd.m0 * nd.inv2;
+    out[K1_VA * (size_t)NODES_MAX + q] = k2 * nd.inv2;
+    out[K1_VC * (size_t)NODES_MAX + q] = i2 * nd.inv2;
 }
 
 // ---------------------------------------------------------------------------------
-// K1b: per sample (one CTA): prefix/suffix sums, node values, Chebyshev and FP32 fits
+// K1b: per sample: prefix/suffix sums, node values, the table's fit.  A lone sample's fit is
+// split over gridDim.y CTAs, each of which repeats the (short) sums and fits its part.
 // ---------------------------------------------------------------------------------
+template <bool LITE>
 __global__ void __launch_bounds__(K1_THREADS)
-table_build_kernel(int B, SampleParams *__restrict__ sp, const double *__restrict__ scratch,
-                   double *__restrict__ tab64, float4 *__restrict__ tab32, int gl8, int max_oct) {
+table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scratch, double *__restrict__ tab64,
+                   float4 *__restrict__ tab32, int max_oct) {
     extern __shared__ double sm[];
+    __shared__ double s_part[2][K1_THREADS / 32];
     const int b = blockIdx.x;
-    if (b >= B) return;
     SampleParams p = sp[b];
     if (p.n_oct > max_oct) {  // never beyond the shared-memory node arrays
         p.n_oct = max_oct;
         __syncthreads();
-        if (threadIdx.x == 0) sp[b].n_oct = max_oct;
+        if (threadIdx.x == 0) sp[b].n_oct = max_oct;  // (every CTA of the sample writes the same)
     }
-    const int NP = gl8 ? LITE_NODES : F64_NODES;  // nodes per FP64 panel
+    constexpr int NP = LITE ? LITE_NODES : F64_NODES;  // nodes per FP64 panel
     const int M = p.n_oct * F64_SUB * NP;
-    double *nodeA = sm;            // [M] interval integrals -> A1 prefix
-    double *nodeC = sm + M;        // [M] interval integrals -> C suffix
-    double *g1s = sm + 2 * M;      // [M]
-    double *g2s = sm + 3 * M;      // [M]
-    const int tid = threadIdx.x;
-    const double alpha = p.alpha, delta = p.delta;
-    const bool stokes = !(alpha > 0.0);
+    double *g1s = sm, *g2s = sm + M;  // [M] node values
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double *t64 = tab64 + (size_t)b * TAB64_STRIDE;
     float4 *t32 = tab32 + (size_t)b * TAB32_STRIDE;
+    const int at = blockIdx.y * K1_THREADS + tid, step = gridDim.y * K1_THREADS;
 
     if (p.status != SWIMMER_OK) {
-        // keep the tables finite so that a stray read cannot produce garbage
-        for (int i = tid; i < TAB64_STRIDE; i += blockDim.x) t64[i] = 0.0;
-        for (int i = tid; i < TAB32_STRIDE; i += blockDim.x) t32[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        // keep the table finite so that a stray read cannot produce garbage
+        if (!LITE)
+            for (int i = at; i < TAB64_STRIDE; i += step) t64[i] = 0.0;
+        else
+            for (int i = at; i < TAB32_STRIDE; i += step) t32[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
     }
+    const double *row = scratch + (size_t)b * K1_SCRATCH;
+    const double tail = row[K1_ROWS * (size_t)NODES_MAX];
 
-    if (!stokes) {
-        const double *IA = scratch + (size_t)b * K1_SCRATCH, *IC = IA + NODES_MAX, *IT = IC + NODES_MAX;
+    if (!(p.alpha > 0.0)) {
         for (int m = tid; m < M; m += blockDim.x) {
-            nodeA[m] = IA[m];
-            nodeC[m] = IC[m];
+            double g1, g2;
+            stokes_g(LITE ? p.delta * sqrt(node6_u(m) - 1.0) : p.delta * g_node[m].sig, p.delta, &g1, &g2);
+            g1s[m] = g1;
+            g2s[m] = g2;
+        }
+    } else if (LITE) {
+        // A1 (prefix) and C (suffix) by warp 0: lanes own contiguous chunks (the order of these
+        // sums is part of what keeps the FP32 tables bit for bit the same)
+        double *nodeA = g1s, *nodeC = g2s;
+        for (int m = tid; m < M; m += K1_THREADS) {
+            nodeA[m] = row[K1_IA * (size_t)NODES_MAX + m];
+            nodeC[m] = m + 1 < M ? row[K1_IC * (size_t)NODES_MAX + m + 1] : tail;
         }
         __syncthreads();
-        if (tid == 0) {
-            double tail = 0.0;
-            for (int k = TAIL_MAX - 1; k >= 0; --k) tail += IT[k];  // far (small) pieces first
-            nodeC[M - 1] = tail;
-        }
-        __syncthreads();
-        // prefix (A1) and suffix (C) sums by warp 0: lanes own contiguous chunks
         if (tid < 32) {
             int chunk = (M + 31) / 32;
             int lo = tid * chunk, hi = min(M, lo + chunk);
@@ -427,64 +729,105 @@ table_build_kernel(int B, SampleParams *__restrict__ sp, const double *__restric
             }
         }
         __syncthreads();
-    }
-
-    // kernel function values at the nodes
-    for (int m = tid; m < M; m += blockDim.x) {
-        double r = delta * sqrt(node_u(m, NP) - 1.0);
-        double g1, g2;
-        if (stokes) {
-            stokes_g(r, delta, &g1, &g2);
-        } else {
-            double x = alpha * r;
-            BesselSet bs = bessel_set(x);
-            double M0 = m0_closed(r, delta), A = nodeA[m], C = nodeC[m];
+        for (int m = tid; m < M; m += K1_THREADS) {
+            double r = p.delta * sqrt(node6_u(m) - 1.0);
+            BesselSet bs;
+            bs.i0 = row[K1_I0 * (size_t)NODES_MAX + m];
+            bs.i2 = row[K1_I2 * (size_t)NODES_MAX + m];
+            bs.k0 = row[K1_K0 * (size_t)NODES_MAX + m];
+            bs.k2 = row[K1_K2 * (size_t)NODES_MAX + m];
+            bs.t2k2 = row[K1_T2K2 * (size_t)NODES_MAX + m];
+            bs.ix2w = row[K1_IX2W * (size_t)NODES_MAX + m];
+            double M0 = m0_closed(r, p.delta), A = nodeA[m], C = nodeC[m];
             double w = 0.5 * (bs.k0 + bs.k2);
-            g1 = bs.ix2w * M0 - w * A - 0.5 * (bs.i0 + bs.i2) * C;
-            g2 = (bs.t2k2 * M0 - bs.k2 * A - bs.i2 * C) / (r * r);
+            double g1 = bs.ix2w * M0 - w * A - 0.5 * (bs.i0 + bs.i2) * C;
+            double g2 = (bs.t2k2 * M0 - bs.k2 * A - bs.i2 * C) / (r * r);
+            g1s[m] = g1;
+            g2s[m] = g2;
         }
-        g1s[m] = g1;
-        g2s[m] = g2;
+    } else {
+        // A1 at node m: sum of the intervals up to it; C: the tail and the intervals beyond it.
+        // Thread t owns the nodes [t chunk, (t + 1) chunk).
+        const double inv_d2 = 1.0 / (p.delta * p.delta);
+        const int chunk = (M + K1_THREADS - 1) / K1_THREADS;
+        const int lo = min(M, tid * chunk), hi = min(M, lo + chunk);
+        double sa = 0.0, sc = 0.0;
+        for (int m = lo; m < hi; ++m) sa += row[K1_IA * (size_t)NODES_MAX + m];
+        for (int m = hi - 1; m >= lo; --m) sc += m + 1 < M ? row[K1_IC * (size_t)NODES_MAX + m + 1] : tail;
+        double pa = sa, pc = sc;  // inclusive scans within the warp (A from the left, C from the right)
+        for (int o = 1; o < 32; o <<= 1) {
+            const double va = __shfl_up_sync(0xffffffffu, pa, o), vc = __shfl_down_sync(0xffffffffu, pc, o);
+            if (lane >= o) pa += va;
+            if (lane + o < 32) pc += vc;
+        }
+        if (lane == 31) s_part[0][warp] = pa;
+        if (lane == 0) s_part[1][warp] = pc;
+        // what lies before (A) and beyond (C) the chunk: the neighbours' inclusive sums, not a
+        // difference (C falls steeply, and inclusive minus own would cancel)
+        const double before = __shfl_up_sync(0xffffffffu, pa, 1), beyond = __shfl_down_sync(0xffffffffu, pc, 1);
+        __syncthreads();
+        double A = 0.0, C = 0.0;
+        for (int k = 0; k < warp; ++k) A += s_part[0][k];
+        for (int k = K1_THREADS / 32 - 1; k > warp; --k) C += s_part[1][k];
+        if (lane > 0) A += before;
+        if (lane < 31) C += beyond;
+        for (int m = lo; m < hi; ++m) {
+            A += row[K1_IA * (size_t)NODES_MAX + m];
+            g1s[m] = A;
+        }
+        for (int m = hi - 1; m >= lo; --m) {
+            C += m + 1 < M ? row[K1_IC * (size_t)NODES_MAX + m + 1] : tail;
+            const double a = g1s[m];
+            g1s[m] = row[K1_E1 * (size_t)NODES_MAX + m] - row[K1_WA * (size_t)NODES_MAX + m] * a -
+                     row[K1_WC * (size_t)NODES_MAX + m] * C;
+            g2s[m] = (row[K1_E2 * (size_t)NODES_MAX + m] - row[K1_VA * (size_t)NODES_MAX + m] * a -
+                      row[K1_VC * (size_t)NODES_MAX + m] * C) * inv_d2;
+        }
     }
     __syncthreads();
 
-    // Chebyshev coefficients per FP64 panel: a_k = (2/n) sum_i g(t_i) T_k(t_i), a_0 halved
-    const int np64 = p.n_oct * F64_SUB;
-    for (int q = tid; q < 2 * np64 * F64_NODES; q += blockDim.x) {
-        int f = q / (np64 * F64_NODES);
-        int rem = q % (np64 * F64_NODES);
-        int panel = rem / F64_NODES, k = rem % F64_NODES;
-        const double *g = (f == 0 ? g1s : g2s) + panel * NP;
-        double s = 0.0;
-        if (NP == F64_NODES) {
+    if (!LITE) {
+        // Chebyshev coefficients per FP64 panel: a_k = (2/n) sum_i g(t_i) T_k(t_i), a_0 halved
+        const int np64 = p.n_oct * F64_SUB;
+        for (int q = at; q < 2 * np64 * F64_NODES; q += step) {  // (a warp shares its row of c_dct)
+            const int f = q / (np64 * F64_NODES), rem = q % (np64 * F64_NODES);
+            const int panel = rem % np64, k = rem / np64;
+            const double *g = (f == 0 ? g1s : g2s) + panel * F64_NODES;
+            double s = 0.0;
             for (int ii = 0; ii < F64_NODES; ++ii) s += g[ii] * c_dct[k][ii];
-        } else if (k < LITE_NODES) {
-            for (int ii = 0; ii < LITE_NODES; ++ii) s += g[ii] * c_dct6[k][ii];
+            t64[(f * F64_PANELS_MAX + panel) * F64_NODES + k] = s;
         }
-        t64[(f * F64_PANELS_MAX + panel) * F64_NODES + k] = s;
+        return;
+    }
+    // Chebyshev coefficients of the 6 node values, in place (each thread its panels)
+    const int np = p.n_oct * F64_SUB;
+    for (int q = tid; q < 2 * np; q += K1_THREADS) {
+        double *g = (q < np ? g1s : g2s) + (q % np) * LITE_NODES, c[LITE_NODES];
+        for (int k = 0; k < LITE_NODES; ++k) {
+            double s = 0.0;
+            for (int ii = 0; ii < LITE_NODES; ++ii) s += g[ii] * c_dct6[k][ii];
+            c[k] = s;
+        }
+        for (int k = 0; k < LITE_NODES; ++k) g[k] = c[k];
     }
     __syncthreads();
-
-    // FP32 quadratic per eighth of an FP64 panel from the FP64 series (Chebyshev fit at 3
-    // nodes, then monomial coefficients in G = 1 + f / F32_SUB, f in [0, 1) across the
-    // panel); the FP32 table holds -g1 (the sign the pair sum's mobility -g1 I + h e e^T
-    // takes) and h = delta^2 g2, for separations measured in units of delta
-    const int np32 = p.n_oct * F32_SUB;
-    constexpr int SPLIT = F32_SUB / F64_SUB;  // FP32 panels per FP64 panel
+    // FP32 quadratic per eighth of an FP64 panel from its series (Chebyshev fit at 3 nodes, then
+    // monomial coefficients in G = 1 + f / F32_SUB, f in [0, 1) across the panel); the FP32 table
+    // holds -g1 (the sign the pair sum's mobility -g1 I + h e e^T takes) and h = delta^2 g2, for
+    // separations measured in units of delta
     float2 *t32b = (float2 *)(t32 + F32_PANELS_MAX);
-    for (int q = tid; q < np32; q += blockDim.x) {
-        int e = q >> F32_SUB_LOG2, jj = q & (F32_SUB - 1);
-        int panel64 = e * F64_SUB + jj / SPLIT;
+    for (int q = at; q < p.n_oct * F32_SUB; q += step) {
+        const int panel = q / F32_SPLIT, jj = q % F32_SPLIT;
         double cf[2][3];
         for (int fn = 0; fn < 2; ++fn) {
-            const double *c = t64 + (fn * F64_PANELS_MAX + panel64) * F64_NODES;
+            const double *c = (fn == 0 ? g1s : g2s) + panel * LITE_NODES;
             double vals[3];
             for (int i = 0; i < 3; ++i) {
                 double f32 = 0.5 * (c_node3[i] + 1.0);  // node of the FP32 panel
-                double f64 = ((jj % SPLIT) + f32) / SPLIT;
+                double f64 = (jj + f32) / F32_SPLIT;
                 double t = 2.0 * f64 - 1.0;
                 double b1 = 0.0, b2 = 0.0;
-                for (int k = F64_DEG; k >= 1; --k) {
+                for (int k = LITE_NODES - 1; k >= 1; --k) {
                     double b0 = 2.0 * t * b1 - b2 + c[k];
                     b2 = b1;
                     b1 = b0;
@@ -605,10 +948,131 @@ static void gauss_legendre(int n, double *x, double *w) {
     }
 }
 
-// constant tables for the table builder (host; constant memory is per device, so once
-// per device)
+// ---- host Bessel functions at the fit's nodes
+// K_0 e^x sqrt(x) and K_1 e^x sqrt(x), x >= 2: the trapezoid rule on the integral representation,
+// whose error decays like exp(-2 pi d/h) for the strip half-width d = acos(1 - 1/x)
+static void host_k_scaled(double x, double *k0, double *k1) {
+    const double d = acos(1.0 - 1.0 / x), h = d / 6.5;
+    double s0 = 0.5, s1 = 0.5;
+    for (int m = 1; m < 4000; ++m) {
+        const double sh = sinh(0.5 * m * h), c1 = 2.0 * sh * sh;  // cosh(m h) - 1
+        const double e = exp(-x * c1);
+        s0 += e;
+        s1 += e * (1.0 + c1);
+        if (e < 1e-19 * s0) break;
+    }
+    *k0 = h * s0 * sqrt(x);
+    *k1 = h * s1 * sqrt(x);
+}
+// I_nu e^-x sqrt(x), nu = 0 or 2, x >= 8: power series to x = 30, Hankel's expansion beyond
+static double host_i_scaled(int nu, double x) {
+    if (x <= 30.0) {
+        const double y = 0.25 * x * x;
+        double term = nu == 0 ? 1.0 : 0.5 * y, s = 0.0;
+        for (int k = 0; k < 200; ++k) {
+            s += term;
+            term *= y / ((k + 1.0) * (k + 1.0 + nu));
+            if (term < 1e-18 * s) break;
+        }
+        return s * exp(-x) * sqrt(x);
+    }
+    const double mu = 4.0 * nu * nu;
+    double s = 1.0, term = 1.0;
+    for (int k = 1; k < 60; ++k) {
+        const double t = -term * (mu - (2.0 * k - 1.0) * (2.0 * k - 1.0)) / (8.0 * k * x);
+        if (fabs(t) > fabs(term)) break;
+        term = t;
+        s += term;
+        if (fabs(term) < 1e-18 * fabs(s)) break;
+    }
+    return s / sqrt(2.0 * PI);
+}
+
+// Chebyshev coefficients in [-1, 1] to powers (in place, n of them)
+static void cheb_to_powers(double *c, int n) {
+    std::vector<double> out(n, 0.0), t0(n, 0.0), t1(n, 0.0), t2(n, 0.0);
+    t0[0] = 1.0;
+    if (n > 1) t1[1] = 1.0;
+    for (int k = 0; k < n; ++k) {
+        const std::vector<double> &tk = k == 0 ? t0 : t1;
+        for (int i = 0; i < n; ++i) out[i] += c[k] * tk[i];
+        if (k >= 1) {
+            for (int i = 0; i < n; ++i) t2[i] = (i ? 2.0 * t1[i - 1] : 0.0) - t0[i];
+            t0 = t1;
+            t1 = t2;
+        }
+    }
+    std::copy(out.begin(), out.end(), c);
+}
+// powers of t = z_scale z + z_shift of f(1/z) on x in [lo, 1/inv_hi], degree deg
+template <class F>
+static void fit_inverse(double lo, double inv_hi, int deg, F f, double *c) {
+    const int n = deg + 1;
+    std::vector<double> v(n);
+    for (int i = 0; i < n; ++i) v[i] = f(z_scale(lo, inv_hi) / (cos(PI * (i + 0.5) / n) - z_shift(lo, inv_hi)));
+    for (int k = 0; k < n; ++k) {
+        double s = 0.0;
+        for (int i = 0; i < n; ++i) s += v[i] * cos(PI * k * (i + 0.5) / n);
+        c[k] = s * (k == 0 ? 1.0 : 2.0) / n;
+    }
+    cheb_to_powers(c, n);
+}
+
+// the sample-independent nodes and quadrature points
+static void build_universal(std::vector<NodeRec> &node, std::vector<QuadRec> &quad, std::vector<int> &at) {
+    const int np = F64_NODES, M = F64_PANELS_MAX * np;
+    std::vector<double> gx[GL_N + 1], gw[GL_N + 1];
+    for (int n = QUAD_MIN; n <= GL_N; ++n) {
+        gx[n].resize(n);
+        gw[n].resize(n);
+        gauss_legendre(n, gx[n].data(), gw[n].data());
+    }
+    double prev = 0.0;
+    at.assign(1, 0);
+    for (int m = 0; m < M; ++m) {
+        const int panel = m / np, i = np - 1 - m % np;  // ascending nodes
+        const double f = 0.5 * (cos(PI * (i + 0.5) / np) + 1.0);
+        const int e = panel >> F64_SUB_LOG2, j = panel & (F64_SUB - 1);
+        // u - 1 without cancellation in the first octave
+        const double um1 = e == 0 ? (j + f) / F64_SUB : ldexp(1.0 + (j + f) / F64_SUB, e) - 1.0;
+        NodeRec r;
+        r.sig = sqrt(um1);
+        r.lns = 0.5 * log(um1);
+        r.rsq = 1.0 / sqrt(r.sig);
+        r.inv2 = 1.0 / um1;
+        const double R = sqrt(1.0 + um1);
+        r.m0 = (um1 / (R + 1.0)) * (R * R + R + 1.0) / (R * R * R) / (2.0 * PI);
+        r.pad = 0.0;
+        node.push_back(r);
+        // the interval's points: enough for 1e-16 in the Bernstein ellipse that reaches s = 0
+        // (ln s; not for the first, which starts there and carries I0 - 1 alone) and s = +-i
+        const double c = 0.5 * (r.sig + prev), hw = 0.5 * (r.sig - prev);
+        double rho = 1e30;
+        if (m > 0) rho = c / hw + sqrt(c / hw * (c / hw) - 1.0);
+        // |z + sqrt(z^2 - 1)| at z = (c + i)/hw by the ellipse's semi-axes sum
+        const double d1 = hypot(c / hw + 1.0, 1.0 / hw), d2 = hypot(c / hw - 1.0, 1.0 / hw), a = 0.5 * (d1 + d2);
+        rho = std::min(rho, a + sqrt(a * a - 1.0));
+        const int n = std::min(GL_N, std::max(QUAD_MIN, (int)ceil(37.0 / (2.0 * log(rho))) + 1));
+        for (int g = n - 1; g >= 0; --g) {  // ascending points
+            QuadRec q;
+            q.sig = c + hw * gx[n][g];
+            q.lns = log(q.sig);
+            q.rsq = 1.0 / sqrt(q.sig);
+            const double R2 = q.sig * q.sig + 1.0;
+            q.w = hw * gw[n][g] * 3.0 * q.sig / (2.0 * PI * R2 * R2 * sqrt(R2));
+            quad.push_back(q);
+        }
+        at.push_back((int)quad.size());
+        prev = r.sig;
+    }
+}
+
+// constant and sample-independent tables for the table builder (host; device memory is per
+// device, so once per device)
 int gl_init() {
     static bool done[256] = {};
+    static std::mutex mutex;
+    std::lock_guard<std::mutex> lock(mutex);
     int dev = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 256) {
@@ -617,58 +1081,72 @@ int gl_init() {
     }
     if (done[dev]) return 0;
     double x[GL_N], w[GL_N];
-    for (int i = 0; i < GL_N; ++i) {
-        double z = cos(PI * (i + 0.75) / (GL_N + 0.5));
-        double dp = 1.0;
-        for (int it = 0; it < 100; ++it) {
-            double p0 = 1.0, p1 = z;
-            for (int k = 2; k <= GL_N; ++k) {
-                double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
-                p0 = p1;
-                p1 = p2;
-            }
-            dp = GL_N * (z * p1 - p0) / (z * z - 1.0);
-            double dz = p1 / dp;
-            z -= dz;
-            if (fabs(dz) < 1e-16) break;
-        }
-        {
-            double p0 = 1.0, p1 = z;
-            for (int k = 2; k <= GL_N; ++k) {
-                double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
-                p0 = p1;
-                p1 = p2;
-            }
-            dp = GL_N * (z * p1 - p0) / (z * z - 1.0);
-        }
-        x[i] = z;
-        w[i] = 2.0 / ((1.0 - z * z) * dp * dp);
-    }
+    gauss_legendre(GL_N, x, w);
     CUDA_TRY(cudaMemcpyToSymbol(c_gl_x, x, sizeof(x)));
     CUDA_TRY(cudaMemcpyToSymbol(c_gl_w, w, sizeof(w)));
-    {
-        double x8[8], w8[8];
-        gauss_legendre(8, x8, w8);
-        CUDA_TRY(cudaMemcpyToSymbol(c_gl8_x, x8, sizeof(x8)));
-        CUDA_TRY(cudaMemcpyToSymbol(c_gl8_w, w8, sizeof(w8)));
+    gauss_legendre(12, x, w);
+    CUDA_TRY(cudaMemcpyToSymbol(c_gl12_x, x, sizeof(double) * 12));
+    CUDA_TRY(cudaMemcpyToSymbol(c_gl12_w, w, sizeof(double) * 12));
+    // Bessel series
+    double i0[SER], i2[SER], k0t[SER_K], t2[SER_K], harmonic[SER_K + 2] = {0.0};
+    for (int k = 1; k < SER_K + 2; ++k) harmonic[k] = harmonic[k - 1] + 1.0 / k;
+    i0[0] = 1.0;
+    i2[0] = 0.5;
+    for (int k = 1; k < SER; ++k) {
+        i0[k] = i0[k - 1] / ((double)k * k);
+        i2[k] = i2[k - 1] / ((double)k * (k + 2.0));
     }
-    double ik[NSER], ikk[2][NSER];
+    for (int k = 0; k < SER_K; ++k) {
+        k0t[k] = harmonic[k] * i0[k];
+        t2[k] = 0.5 * (harmonic[k] + harmonic[k + 2]) * i2[k];
+    }
+    CUDA_TRY(cudaMemcpyToSymbol(c_i0, i0, sizeof(i0)));
+    CUDA_TRY(cudaMemcpyToSymbol(c_i2, i2, sizeof(i2)));
+    CUDA_TRY(cudaMemcpyToSymbol(c_k0t, k0t, sizeof(k0t)));
+    CUDA_TRY(cudaMemcpyToSymbol(c_t2, t2, sizeof(t2)));
+    // Bessel fits in 1/x
+    double pk[2][2][DEG_K + 1], pi1[2][DEG_I1 + 1], pi2[2][DEG_I2 + 1];
+    for (int nu = 0; nu < 2; ++nu) {
+        auto k = [nu](double v) {
+            double a, b;
+            host_k_scaled(v, &a, &b);
+            return nu == 0 ? a : b;
+        };
+        fit_inverse(2.0, 1.0 / K_SPLIT, DEG_K, k, pk[nu][0]);
+        fit_inverse(K_SPLIT, 0.0, DEG_K, k, pk[nu][1]);
+        auto i = [nu](double v) { return host_i_scaled(2 * nu, v); };
+        fit_inverse(I_SERIES, 1.0 / I_SPLIT, DEG_I1, i, pi1[nu]);
+        fit_inverse(I_SPLIT, 0.0, DEG_I2, i, pi2[nu]);
+    }
+    CUDA_TRY(cudaMemcpyToSymbol(c_k0, pk[0], sizeof(pk[0])));
+    CUDA_TRY(cudaMemcpyToSymbol(c_k1, pk[1], sizeof(pk[1])));
+    CUDA_TRY(cudaMemcpyToSymbol(c_i0p, pi1[0], sizeof(pi1[0])));
+    CUDA_TRY(cudaMemcpyToSymbol(c_i2p, pi1[1], sizeof(pi1[1])));
+    CUDA_TRY(cudaMemcpyToSymbol(c_i0q, pi2[0], sizeof(pi2[0])));
+    CUDA_TRY(cudaMemcpyToSymbol(c_i2q, pi2[1], sizeof(pi2[1])));
+    // table fits
+    double dct[F64_NODES][F64_NODES];
+    for (int ii = 0; ii < F64_NODES; ++ii) {
+        int i = F64_NODES - 1 - ii;  // ascending node ii is Chebyshev index i
+        for (int k = 0; k < F64_NODES; ++k)
+            dct[k][ii] = (2.0 / F64_NODES) * cos(PI * k * (i + 0.5) / F64_NODES) * (k == 0 ? 0.5 : 1.0);
+    }
+    CUDA_TRY(cudaMemcpyToSymbol(c_dct, dct, sizeof(dct)));
+    // FP32 handles
+    double ik[NSER], ikk[2][NSER], hk[HARM];
     for (int k = 0; k < NSER; ++k) {
         ik[k] = k ? 1.0 / k : 0.0;
         ikk[0][k] = 1.0 / ((k + 1.0) * (k + 1.0));
         ikk[1][k] = 1.0 / ((k + 1.0) * (k + 3.0));
     }
+    hk[0] = 0.0;
+    for (int k = 1; k < HARM; ++k) hk[k] = hk[k - 1] + ik[k];
     CUDA_TRY(cudaMemcpyToSymbol(c_inv_k, ik, sizeof(ik)));
     CUDA_TRY(cudaMemcpyToSymbol(c_inv_kk, ikk, sizeof(ikk)));
-    double ct[F64_NODES], dct[F64_NODES][F64_NODES];
-    for (int ii = 0; ii < F64_NODES; ++ii) {
-        int i = F64_NODES - 1 - ii;  // ascending node ii is Chebyshev index i
-        ct[ii] = cos(PI * (i + 0.5) / F64_NODES);
-        for (int k = 0; k < F64_NODES; ++k)
-            dct[k][ii] = (2.0 / F64_NODES) * cos(PI * k * (i + 0.5) / F64_NODES) * (k == 0 ? 0.5 : 1.0);
-    }
-    CUDA_TRY(cudaMemcpyToSymbol(c_cheb_t, ct, sizeof(ct)));
-    CUDA_TRY(cudaMemcpyToSymbol(c_dct, dct, sizeof(dct)));
+    CUDA_TRY(cudaMemcpyToSymbol(c_harm, hk, sizeof(hk)));
+    gauss_legendre(8, x, w);
+    CUDA_TRY(cudaMemcpyToSymbol(c_gl8_x, x, sizeof(double) * 8));
+    CUDA_TRY(cudaMemcpyToSymbol(c_gl8_w, w, sizeof(double) * 8));
     double ct6[LITE_NODES], dct6[LITE_NODES][LITE_NODES];
     for (int ii = 0; ii < LITE_NODES; ++ii) {
         int i = LITE_NODES - 1 - ii;
@@ -685,6 +1163,18 @@ int gl_init() {
     }
     CUDA_TRY(cudaMemcpyToSymbol(c_node3, n3, sizeof(n3)));
     CUDA_TRY(cudaMemcpyToSymbol(c_dct3, d3, sizeof(d3)));
+    // FP64 handles: nodes and quadrature points
+    std::vector<NodeRec> node;
+    std::vector<QuadRec> quad;
+    std::vector<int> at;
+    build_universal(node, quad, at);
+    if (quad.size() > QUAD_CAP) {
+        set_error("the table build's quadrature needs %zu points", quad.size());
+        return SWIMMER_E_ARG;
+    }
+    CUDA_TRY(cudaMemcpyToSymbol(g_node, node.data(), sizeof(NodeRec) * node.size()));
+    CUDA_TRY(cudaMemcpyToSymbol(g_quad, quad.data(), sizeof(QuadRec) * quad.size()));
+    CUDA_TRY(cudaMemcpyToSymbol(g_quad_at, at.data(), sizeof(int) * at.size()));
     done[dev] = true;
     return 0;
 }
@@ -710,21 +1200,35 @@ int launch_prepare(swimmer_handle *h, int B, const double *theta, const int *n_p
     return 0;
 }
 
+// the two table kernels on B samples whose scratch rows start at `scratch`
+static int table_kernels(int B, SampleParams *sp, double *scratch, double *tab64, float4 *tab32, bool lite, int oct,
+                         int sms, cudaStream_t s) {
+    const int M = oct * F64_SUB * (lite ? LITE_NODES : F64_NODES);
+    const dim3 ga(B, (M + K1A_THREADS - 1) / K1A_THREADS + 1);
+    table_nodes_kernel<<<ga, K1A_THREADS, 0, s>>>(sp, scratch, lite ? 1 : 0, oct);
+    CUDA_TRY(cudaGetLastError());
+    // the fit of few samples over several CTAs each (at most one per octave)
+    const dim3 gb(B, std::max(1, std::min(oct, sms / B)));
+    const size_t smem = 2 * (size_t)M * sizeof(double);
+    if (lite)
+        table_build_kernel<true><<<gb, K1_THREADS, smem, s>>>(sp, scratch, tab64, tab32, oct);
+    else
+        table_build_kernel<false><<<gb, K1_THREADS, smem, s>>>(sp, scratch, tab64, tab32, oct);
+    CUDA_TRY(cudaGetLastError());
+    return 0;
+}
+
 int launch_table_build(swimmer_handle *h, int B, int need64, cudaStream_t s) {
     // node arrays for the handle's octaves (kernel_eval may need the full range)
-    // need64: 0 = FP32 handle build, 1 = FP64 build, 2/3 = the same over the full range
+    // need64: 0 = FP32 table, 1 = FP64 table, 2/3 = FP64 / FP32 table over the full range
     const int oct = need64 >= 2 ? N_OCT_MAX : handle_octaves(h);
     const bool lite = need64 == 0 || need64 == 3;
-    const int M = oct * F64_SUB * (lite ? LITE_NODES : F64_NODES);
-    size_t smem = 4 * (size_t)M * sizeof(double);
-    CUDA_TRY(cudaFuncSetAttribute(table_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)(4 * (size_t)NODES_MAX * sizeof(double))));
-    dim3 ga(B, (M + TAIL_MAX + K1A_THREADS - 1) / K1A_THREADS);
-    table_integrals_kernel<<<ga, K1A_THREADS, 0, s>>>(B, h->sp, h->k1_scratch, lite ? 1 : 0, oct);
-    CUDA_TRY(cudaGetLastError());
-    table_build_kernel<<<B, K1_THREADS, smem, s>>>(B, h->sp, h->k1_scratch, h->tab64, h->tab32, lite ? 1 : 0, oct);
-    CUDA_TRY(cudaGetLastError());
-    prof_count(h, 2);
+    for (int b = 0; b < B; b += K1_SLICE) {  // the scratch holds K1_SLICE samples
+        int rc = table_kernels(std::min(K1_SLICE, B - b), h->sp + b, h->k1_scratch, h->tab64 + (size_t)b * TAB64_STRIDE,
+                               h->tab32 + (size_t)b * TAB32_STRIDE, lite, oct, h->num_sms, s);
+        if (rc) return rc;
+        prof_count(h, 2);
+    }
     return 0;
 }
 
@@ -748,7 +1252,7 @@ int launch_kernel_eval(swimmer_handle *h, int m, const double *r, double *g1, do
 // budget at start-up and must not grow it per request.  For them the
 // table build of one sample (the kernels above that use scratch memory) runs on scratch
 // that lives in file-scope device arrays: every GPU that loads this library holds these
-// ~98 KB until the process exits, and every call on a device shares them.
+// ~0.2 MB until the process exits, and every call on a device shares them.
 namespace {
 __device__ __align__(256) double g_noalloc_scratch[K1_SCRATCH];
 __device__ __align__(256) double g_noalloc_tab64[TAB64_STRIDE];
@@ -776,14 +1280,13 @@ int noalloc_setup(int dev, NoallocPtrs *out) {
         CUDA_TRY(cudaGetSymbolAddress((void **)&p.tab64, g_noalloc_tab64));
         CUDA_TRY(cudaGetSymbolAddress((void **)&p.tab32, g_noalloc_tab32));
         CUDA_TRY(cudaGetSymbolAddress((void **)&p.sp, g_noalloc_sp));
-        CUDA_TRY(cudaFuncSetAttribute(table_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(4 * (size_t)NODES_MAX * sizeof(double))));
         // load every kernel of the call now: with lazy module loading a kernel first launched
         // later (kernel_eval_kernel after calls with m = 0) would load its code then
         cudaFuncAttributes fa;
         CUDA_TRY(cudaFuncGetAttributes(&fa, set_sample_kernel));
-        CUDA_TRY(cudaFuncGetAttributes(&fa, table_integrals_kernel));
-        CUDA_TRY(cudaFuncGetAttributes(&fa, table_build_kernel));
+        CUDA_TRY(cudaFuncGetAttributes(&fa, table_nodes_kernel));
+        CUDA_TRY(cudaFuncGetAttributes(&fa, table_build_kernel<false>));
+        CUDA_TRY(cudaFuncGetAttributes(&fa, table_build_kernel<true>));
         CUDA_TRY(cudaFuncGetAttributes(&fa, kernel_eval_kernel));
         p.ready = true;
     }
@@ -809,15 +1312,10 @@ extern "C" int swimmer_kernel_eval_noalloc(double alpha, double delta, double r_
     if (rc) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     const bool lite = precision != SWIMMER_FP64;  // as FP32 handles build their table
-    const int M = N_OCT_MAX * F64_SUB * (lite ? LITE_NODES : F64_NODES);
     set_sample_kernel<<<1, 1, 0, s>>>(p.sp, alpha, delta, r_max);
     CUDA_TRY(cudaGetLastError());
-    dim3 ga(1, (M + TAIL_MAX + K1A_THREADS - 1) / K1A_THREADS);
-    table_integrals_kernel<<<ga, K1A_THREADS, 0, s>>>(1, p.sp, p.scratch, lite ? 1 : 0, N_OCT_MAX);
-    CUDA_TRY(cudaGetLastError());
-    table_build_kernel<<<1, K1_THREADS, 4 * (size_t)M * sizeof(double), s>>>(1, p.sp, p.scratch, p.tab64, p.tab32,
-                                                                           lite ? 1 : 0, N_OCT_MAX);
-    CUDA_TRY(cudaGetLastError());
+    rc = table_kernels(1, p.sp, p.scratch, p.tab64, p.tab32, lite, N_OCT_MAX, N_OCT_MAX, s);
+    if (rc) return rc;
     if (m > 0) {
         kernel_eval_kernel<<<(m + 127) / 128, 128, 0, s>>>(m, r, g1, g2, p.sp, p.tab64, p.tab32, precision);
         CUDA_TRY(cudaGetLastError());
