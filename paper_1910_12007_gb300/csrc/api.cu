@@ -156,10 +156,11 @@ extern "C" int swimmer_init(const swimmer_config *cfg, swimmer_handle **out) {
     CUDA_TRY(cudaDeviceGetAttribute(&h->max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     CUDA_TRY(cudaDeviceGetAttribute(&h->regs_per_sm, cudaDevAttrMaxRegistersPerMultiprocessor, h->device));
     const int B = cfg->b_max;
-    ALLOC(h->tab64, (size_t)B * TAB64_STRIDE);
+    ALLOC(h->tab64, (size_t)(cfg->precision == SWIMMER_FP64 ? B : 1) * TAB64_STRIDE);
     ALLOC(h->k1_scratch, (size_t)std::min(B, K1_SLICE) * K1_SCRATCH);
     ALLOC(h->tab32, (size_t)B * TAB32_STRIDE);
-    ALLOC(h->pq, (size_t)B * cfg->n_max);
+    // (FP32 handles keep float2)
+    ALLOC(h->pq, cfg->precision == SWIMMER_FP64 ? (size_t)B * cfg->n_max : ((size_t)B * cfg->n_max + 1) / 2);
     ALLOC(h->sp, B);
     ALLOC(h->order, B);
     ALLOC(h->queue, 4);
@@ -211,6 +212,7 @@ extern "C" int swimmer_init(const swimmer_config *cfg, swimmer_handle **out) {
         }
     }
     rc = gl_init();
+    if (!rc) rc = pressure_init();
     if (!rc) rc = upload_pair_units(h);
     if (!rc) rc = tmcmc_templates_init(h);
     if (rc) {

@@ -11,17 +11,21 @@
 // octave cut into equal panels.  The kernel functions are analytic in u except at u = 0,
 // so short panels far from 0 make low-degree polynomials accurate.
 constexpr int N_OCT_MAX = 24;          // u < 2^24 (r/delta < 4096)
-constexpr int F64_SUB_LOG2 = 3;        // 8 panels per octave
+constexpr int F64_SUB_LOG2 = 3;        // the table build's panels: 8 per octave
 constexpr int F64_SUB = 1 << F64_SUB_LOG2;
-constexpr int F64_DEG = 9;             // Chebyshev degree 9 per panel (10 nodes)
+constexpr int F64_DEG = 9;             // degree 9 per build panel (10 nodes)
 constexpr int F64_NODES = F64_DEG + 1;
 constexpr int F32_SUB_LOG2 = 6;        // 64 panels per octave (quadratic)
 constexpr int F32_SUB = 1 << F32_SUB_LOG2;
 constexpr int F64_PANELS_MAX = N_OCT_MAX * F64_SUB;
 constexpr int F32_PANELS_MAX = N_OCT_MAX * F32_SUB;
 constexpr int NODES_MAX = F64_PANELS_MAX * F64_NODES;   // 1920
-// FP64 table per sample: [2][F64_PANELS_MAX][F64_NODES] Chebyshev coefficients
-constexpr int TAB64_STRIDE = 2 * F64_PANELS_MAX * F64_NODES;
+// FP64 table per sample: one record of F64_REC float4 per panel, 32 panels per octave
+// (table_eval.cuh)
+constexpr int F64_FINE_LOG2 = 5;
+constexpr int F64_FINE = 1 << F64_FINE_LOG2;
+constexpr int F64_REC = 7;
+constexpr int TAB64_STRIDE = N_OCT_MAX * F64_FINE * F64_REC;
 // FP32 table per sample (float4 units): part A [F32_PANELS_MAX] float4 = (g1 c0, g1 c1,
 // g1 c2, h c0) then part B [F32_PANELS_MAX] float2 = (h c1, h c2), h = delta^2 g2: monomial
 // quadratic coefficients in G = 1 + f / F32_SUB, f in [0, 1) the local panel coordinate
@@ -105,10 +109,10 @@ struct swimmer_handle {
     int max_smem;  // opt-in shared memory per block (bytes)
     int regs_per_sm;  // 32-bit registers per SM
     // per-sample workspace (b_max samples)
-    double *tab64;          // [b_max][TAB64_STRIDE]
+    float4 *tab64;          // [b_max][TAB64_STRIDE] (FP32 handles: one, for kernel_eval and flow)
     double *k1_scratch;     // [min(b_max, K1_SLICE)][K1_SCRATCH] node values of the table build
     float4 *tab32;          // [b_max][TAB32_STRIDE]
-    float2 *pq;             // [b_max][n_max] FP32 kernel: preferred-curvature coefficients
+    double2 *pq;            // [b_max][n_max] preferred-curvature coefficients (FP32 handles: as float2)
     SampleParams *sp;       // [b_max]
     int *order;             // [b_max] processing order (longest first)
     int *queue;             // [4] work counters
@@ -186,6 +190,7 @@ int upload_pair_units(swimmer_handle *h);
 int launch_kernel_eval(swimmer_handle *h, int m, const double *r, double *g1, double *g2,
                        int precision, cudaStream_t s);
 int gl_init();
+int pressure_init();
 // octaves the tables need for the largest sample a handle serves
 int handle_octaves(const swimmer_handle *h);
 int launch_set_sample(swimmer_handle *h, double alpha, double delta, double r_max, cudaStream_t s);

@@ -14,7 +14,7 @@
 //   C  point forces F = -dE/dX (Eq. Fenergy) gathered from the stencils;
 //   D  Brinkmanlet pair sum (Eq. BrV) v_i = (1/mu) sum_j [-F_j g1 + (F_j . d) d g2],
 //      d = X_i - X_j, with g1, g2 from the per-sample shared-memory table (quadratic in
-//      G = 1 + f/64 in FP32, Chebyshev degree 9 in FP64).
+//      G = 1 + f/64 in FP32; in FP64 degree 7, all but its leading term in pairs of floats).
 //      FP32: every unordered pair once.  g1, g2 and (F . d) d are even in d, so one table
 //      lookup serves v_i and v_j.  The points form blocks of 32; a warp takes a block pair
 //      (I, J) along diagonals: lane l holds target I*32 + l and meets source
@@ -31,8 +31,8 @@
 //      in a fixed order with TwoSum, so results do not depend on scheduling.  Launches
 //      whose shared memory holds an SM to one CTA of at most 512 threads use an
 //      instantiation compiled for 128 registers a thread.
-//      FP64: target i meets source i + d at step d (the point list stored twice), the S
-//      threads of a target splitting the sources and combining with warp shuffles;
+//      FP64: target i meets source i + d mod n at step d, the S threads of a target splitting
+//      the sources and combining with warp shuffles;
 //   E  forward Euler X += dt v: FP64 positions in the FP64 kernel, double-float (hi + lo
 //      FP32, about 48 significant bits) positions updated by TwoSum in the FP32 kernel;
 //      every obs_every steps the head point is compared with the observations and the
@@ -57,9 +57,9 @@ struct FwdArgs {
     const SampleParams *sp;
     const int *order;
     int *queue;
-    const double *tab64;
+    const float4 *tab64;
     const float4 *tab32;
-    float2 *pq;  // FP32 kernel: [B][n_max] preferred-curvature coefficients (P_k, Q_k) per run
+    void *pq;  // [B][n_max] preferred-curvature coefficients (P_k, Q_k) per run (float2 or double2)
     double mu, dt, kt, eta, omega;
     double hr_over_ds, gap_over_ds, k_head_tens, k_head_c, k_neck_tens, k_neck_ang;  // head model
     int obs_kind;
@@ -132,7 +132,7 @@ struct RestF32 {
     float l0, l02_hi, l02_lo, inv_l02, k2;
 };
 struct RestF64 {
-    double l0, inv_l02, k2;
+    double l0, inv_l02, k2_l0;
 };
 
 __host__ __device__ inline RestF32 rest_f32(double l0, double k) {
@@ -149,7 +149,7 @@ __host__ __device__ inline RestF64 rest_f64(double l0, double k) {
     RestF64 r;
     r.l0 = l0;
     r.inv_l02 = 1.0 / (l0 * l0);
-    r.k2 = 2.0 * k;
+    r.k2_l0 = 2.0 * k / l0;
     return r;
 }
 
@@ -181,20 +181,20 @@ __device__ __forceinline__ double spring_f64(const double *sx, const double *sy,
                                              double &ex, double &ey, double &strain) {
     ex = sx[j] - sx[i];
     ey = sy[j] - sy[i];
-    double s2 = fma(fma(ex, ex, ey * ey), r.inv_l02, -1.0);  // l^2/l0^2 - 1
-    strain = s2 / (1.0 + sqrt(1.0 + s2));
-    double ell = r.l0 * (1.0 + strain);
-    return r.k2 * strain / ell;
+    const double s2 = fma(fma(ex, ex, ey * ey), r.inv_l02, -1.0);  // l^2/l0^2 - 1
+    const double rs = rsqrt(1.0 + s2);                             // l0/l
+    strain = s2 / fma(1.0 + s2, rs, 1.0);
+    return r.k2_l0 * strain * rs;
 }
 
 // table region in shared memory: FP32: float4 part A [P] then float2 part B [P] (24 bytes a
 // panel), or with MERGED one 32-byte record per panel [P][2] float4, so that one address serves
 // both loads of a lookup (the 128-register instantiation, whose launches are held to one or two
 // CTAs per SM by other limits, so the larger table costs no occupancy there);
-// FP64: Chebyshev coefficients of g1 [P][10] then of g2 [P][10]
+// FP64: the panels' records (table_eval.cuh)
 template <bool F64, bool MERGED = false>
 __host__ __device__ size_t table_bytes(int P) {
-    return F64 ? sizeof(double) * 2 * P * F64_NODES : (MERGED ? 2 * sizeof(float4) : sizeof(float4) + sizeof(float2)) * P;
+    return F64 ? sizeof(float4) * P * F64_REC : (MERGED ? 2 * sizeof(float4) : sizeof(float4) + sizeof(float2)) * P;
 }
 
 __host__ __device__ inline size_t align32(size_t b) { return (b + 31) & ~size_t(31); }
@@ -210,8 +210,8 @@ __host__ __device__ inline int pair_warps(int n_max, int threads) {
 }
 
 // Per-step state in shared memory.
-// FP64: positions sx, sy [n_max] (double); sources (x, y, Fx, Fy) [2 n_max] (the point list
-//   twice in a row); tension vectors tx, ty [n_max]; six bending terms [6][n_max].
+// FP64: positions sx, sy [n_max] (double); sources (x, y, Fx, Fy) [n_max]; tension vectors
+//   tx, ty [n_max]; six bending terms [6][n_max].
 // FP32: positions xh, xl, yh, yl [n_max]; sources per block of 32 points as two planes of
 //   pair records ([nbm][2][32] float4, plane_a / plane_b); tension vectors and bending terms
 //   [8][n_max], which
@@ -219,7 +219,7 @@ __host__ __device__ inline int pair_warps(int n_max, int threads) {
 //   instead, the region growing when those need more room.
 template <bool F64>
 __host__ __device__ size_t state_bytes(int n_max, int threads) {
-    if (F64) return align32(16 * (size_t)n_max) + 2 * 32 * (size_t)n_max + 8 * 8 * (size_t)n_max;
+    if (F64) return align32(16 * (size_t)n_max) + 32 * (size_t)n_max + 8 * 8 * (size_t)n_max;
     const size_t nbm = (n_max + 31) / 32;
     size_t forces = 32 * (size_t)n_max, part = 256 * nbm * (size_t)pair_warps(n_max, threads);
     // (the same bytes are the pair-unit assignment's scratch at the start of a sample)
@@ -438,8 +438,8 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
     double *sy = sx + n_max;
     float *xh = (float *)smraw, *xl = xh + n_max, *yh = xl + n_max, *yl = yh + n_max;
     const int nbm = (n_max + 31) >> 5;
-    R4 *src = (R4 *)(smraw + align32(16 * (size_t)n_max));  // FP64 [2 n_max]; FP32 [nbm][64]
-    R *tvx = (R *)(src + (F64 ? 2 * n_max : 64 * nbm));    // tension vectors, then bending
+    R4 *src = (R4 *)(smraw + align32(16 * (size_t)n_max));  // FP64 [n_max]; FP32 [nbm][64]
+    R *tvx = (R *)(src + (F64 ? n_max : 64 * nbm));    // tension vectors, then bending
     R *tvy = tvx + n_max;
     R *bend = tvy + n_max;  // [6][n_max]
     float2 *part = (float2 *)tvx;  // FP32 pair sum: per-warp partial velocities
@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
     // FP32 kernel: (cos, sin)(omega t) of the current step, and the FP64 rotation state
     // (cos, sin)(omega step dt), (cos, sin)(omega dt) that thread 0 advances once per step
     __shared__ float s_rot[2];
-    __shared__ double s_rot64[4];
+    __shared__ double s_rot64[F64 ? 64 : 4];  // FP64 kernel: (cos, sin)(omega t) of 32 steps
     // FP32 pair sum: warp w processes units [s_wstart[w], s_wstart[w + 1]) of the sample's list
     __shared__ int s_wstart[F64 ? 1 : 33];
     static_assert(F_COUNT <= 16, "s_f32 holds 16 constants");
@@ -492,14 +492,11 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
         }
         // ---- table into shared memory
         const int P = a.tab_panels;
-        const int npan = min(P, p.n_oct * (F64 ? F64_SUB : F32_SUB));
+        const int npan = min(P, p.n_oct * (F64 ? F64_FINE : F32_SUB));
         if (F64) {
-            const double *g = a.tab64 + (size_t)b * TAB64_STRIDE;
-            double *t = (double *)tabraw;
-            for (int i = tid; i < npan * F64_NODES; i += T) {
-                t[i] = g[i];
-                t[(size_t)P * F64_NODES + i] = g[F64_PANELS_MAX * F64_NODES + i];
-            }
+            const float4 *g = a.tab64 + (size_t)b * TAB64_STRIDE;
+            float4 *t = (float4 *)tabraw;
+            for (int i = tid; i < npan * F64_REC; i += T) t[i] = g[i];
         } else {
             const float4 *g = a.tab32 + (size_t)b * TAB32_STRIDE;
             const float2 *gb = (const float2 *)(g + F32_PANELS_MAX);
@@ -608,17 +605,21 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
             s_rot[0] = 1.f;
             s_rot[1] = 0.f;
         }
-        if (!F64) {
+        {
             // the preferred curvature of flagellum point k (Appendix: y^ = a (1 - s/L)
             // sin(eta s - omega t), zeta^ = d^2 y^/ds^2) split as
             // zeta^_k(t) = P_k cos(omega t) + Q_k sin(omega t), made in FP64 once per run
-            float2 *pq = a.pq + (size_t)b * n_max;
+            const size_t row = (size_t)b * n_max;
             for (int k = tid; k < nf; k += T) {
                 const double sk = k * ds;
                 double sn, cs;
                 sincos(a.eta * sk, &sn, &cs);
                 const double c1 = 2.0 * a.eta / L, c2 = (1.0 - sk / L) * a.eta * a.eta;
-                pq[k] = make_float2((float)(-p.amp * (c1 * cs + c2 * sn)), (float)(-p.amp * (c1 * sn - c2 * cs)));
+                const double pk = -p.amp * (c1 * cs + c2 * sn), qk = -p.amp * (c1 * sn - c2 * cs);
+                if (F64)
+                    ((double2 *)a.pq)[row + k] = make_double2(pk, qk);
+                else
+                    ((float2 *)a.pq)[row + k] = make_float2((float)pk, (float)qk);
             }
         }
         const double dt_mu = a.dt / a.mu;
@@ -643,10 +644,9 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
         if (!F64 && tid == 0)
             assign_units((unsigned *)(tabraw + table_bytes<F64, MERGED>(P)), n_units, n_pw, (unsigned *)part, s_wstart);
         __syncthreads();
-        const R r_ds = F64 ? (R)ds : (R)s_f32[F_DS], r_inv2ds = F64 ? (R)(0.5 / ds) : (R)s_f32[F_INV2DS];
+        const R r_inv2ds = F64 ? (R)(0.5 / ds) : (R)s_f32[F_INV2DS];
         const R r_invds2 = F64 ? (R)(1.0 / (ds * ds)) : (R)s_f32[F_INVDS2];
         const R kc2ds = F64 ? (R)(2.0 * p.kc * ds) : (R)s_f32[F_KC2DS];
-        const R r_amp = (R)p.amp, r_eta = (R)a.eta, r_omega = (R)a.omega, r_L = (R)L;  // (FP64 kernel)
         const R inv_d2 = (R)(1.0 / (p.delta * p.delta));
         if (vel_obs(a, nh) && tid < 32) {  // head centre at the previous observation
             double cx, cy;
@@ -671,7 +671,10 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
         const int obs_every = (int)min(a.obs_every, (long long)INT_MAX);  // > steps: no observation
         int obs_left = obs_every, obs_idx = 0;
         for (int step = 0; step < (int)last; ++step) {
-            const double tR = (double)step * a.dt;  // (FP64 kernel; the FP32 kernel rotates s_rot)
+            if (F64 && (step & 31) == 0) {  // (the last reads of s_rot64 lie before a barrier)
+                if (tid >= T - 32) sincos(a.omega * ((double)(step + lane) * a.dt), &s_rot64[2 * lane + 1], &s_rot64[2 * lane]);
+                __syncthreads();
+            }
             const bool obs_step = --obs_left == 0;
             int bad = 0;
             // ---- A+B: segments, tension, curvature stencils, relative positions.  Thread k
@@ -735,11 +738,9 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                     tvx[k] = tk * epx;
                     tvy[k] = tk * epy;
                 }
-                if (F64) {  // the point list stored twice
+                if (F64) {
                     src[k].x = qx;
                     src[k].y = qy;
-                    src[k + n].x = qx;
-                    src[k + n].y = qy;
                 } else {  // plane A: own entry, and the previous entry's second half
                     const int ka = plane_a(k), kp = plane_a(plane_prev(k));
                     src[ka].x = qx;
@@ -754,7 +755,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                     R S2 = A * A + Bv * Bv;
                     R rs;
                     if (F64) {
-                        rs = (R)(1.0 / sqrt((double)S2));
+                        rs = (R)rsqrt((double)S2);
                     } else {
                         // the hardware estimate plus one Newton step: its ~2 ulp error would
                         // otherwise enter zeta and the stencils, which multiply it by 1/ds^2
@@ -769,16 +770,14 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                     if (hd) {
                         zhat = (R)s_model[M_IHR];  // preferred head curvature 1/H_r
                     } else {
+                        // zeta^_k(t) = P_k cos(omega t) + Q_k sin(omega t), P and Q made in FP64 for
+                        // the run.  FP64: the cosines and sines of 32 steps at a time, a lane each;
+                        // FP32: rotated in FP64 once per step
                         if (F64) {
-                            const R s = (R)kl * r_ds;
-                            const R ph = r_eta * s - r_omega * tR;
-                            double sd, cd;
-                            sincos((double)ph, &sd, &cd);
-                            zhat = -r_amp * ((R)2 * r_eta / r_L * (R)cd + ((R)1 - s / r_L) * r_eta * r_eta * (R)sd);
+                            const double2 c = ((const double2 *)a.pq)[(size_t)b * n_max + kl];
+                            zhat = (R)fma(c.x, s_rot64[2 * (step & 31)], c.y * s_rot64[2 * (step & 31) + 1]);
                         } else {
-                            // zeta^_k(t) = P_k cos(omega t) + Q_k sin(omega t) (made in FP64 for the
-                            // run); (cos, sin)(omega t) is advanced in FP64 once per step
-                            const float2 c = a.pq[(size_t)b * n_max + kl];
+                            const float2 c = ((const float2 *)a.pq)[(size_t)b * n_max + kl];
                             zhat = (R)fmaf(c.x, s_rot[0], c.y * s_rot[1]);
                         }
                     }
@@ -914,8 +913,6 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 if (F64) {
                     src[k].z = fx;
                     src[k].w = fy;
-                    src[k + n].z = fx;
-                    src[k + n].w = fy;
                 } else {  // plane B
                     const int kb = plane_b(k), kp = plane_b(plane_prev(k));
                     src[kb].x = fx;
@@ -942,15 +939,18 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 if (tgt < n) {
                     const R4 me = src[tgt];
                     const double xi = (double)me.x, yi = (double)me.y;
-                    const double *tab = (const double *)tabraw;
+                    const float4 *tab = (const float4 *)tabraw;
                     double vx = 0.0, vy = 0.0;
-                    const R4 *sp = src + tgt + split;
-                    for (int d = split; d < n; d += S, sp += S) {
-                        R4 q = *sp;
+                    int j = tgt + split;
+                    if (j >= n) j -= n;
+                    for (int d = split; d < n; d += S) {
+                        const R4 q = src[j];
+                        j += S;
+                        if (j >= n) j -= n;
                         double dx = xi - (double)q.x, dy = yi - (double)q.y;
                         double u = fma(fma(dx, dx, dy * dy), (double)inv_d2, 1.0);
                         double g1, g2;
-                        kern_f64(tab, P, npan - 1, u, g1, g2);
+                        kern_f64(tab, npan - 1, u, g1, g2);
                         double fd = fma((double)q.z, dx, (double)q.w * dy);
                         double wv = fd * g2;
                         vx = fma(wv, dx, fma(-(double)q.z, g1, vx));
@@ -1287,7 +1287,7 @@ int upload_pair_units(swimmer_handle *h) {
 // the sample size.  The autotuned choice wins.
 bool forward_fits(const swimmer_handle *h, int threads, int precision) {
     const bool f64 = precision == SWIMMER_FP64;
-    const int P = handle_octaves(h) * (f64 ? F64_SUB : F32_SUB);
+    const int P = handle_octaves(h) * (f64 ? F64_FINE : F32_SUB);
     size_t smem = f64 ? smem_bytes<true>(h->cfg.n_max, P, threads) : smem_bytes<false>(h->cfg.n_max, P, threads);
     return smem + 1024 <= (size_t)h->max_smem;  // static shared memory of the kernel
 }
@@ -1297,7 +1297,7 @@ bool forward_fits(const swimmer_handle *h, int threads, int precision) {
 int forward_slots(const swimmer_handle *h, int precision) {
     const bool f64 = precision == SWIMMER_FP64;
     const int T = forward_min_threads(h, precision);
-    const int P = handle_octaves(h) * (f64 ? F64_SUB : F32_SUB);
+    const int P = handle_octaves(h) * (f64 ? F64_FINE : F32_SUB);
     size_t smem = f64 ? smem_bytes<true>(h->cfg.n_max, P, T) : smem_bytes<false>(h->cfg.n_max, P, T);
     auto kern = forward_kernel_for(f64, h->cfg);
     int per_sm = 0;
@@ -1390,7 +1390,7 @@ int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, do
     const bool f64 = precision == SWIMMER_FP64;
     a.units = h->units;
     a.mode = f64 ? 0 : (shape & SHAPE_QUAD) ? 2 : (shape & SHAPE_WIDE) ? 1 : 0;
-    a.tab_panels = handle_octaves(h) * (f64 ? F64_SUB : F32_SUB);
+    a.tab_panels = handle_octaves(h) * (f64 ? F64_FINE : F32_SUB);
     size_t smem = f64 ? smem_bytes<true>(a.n_max, a.tab_panels, T) : smem_bytes<false>(a.n_max, a.tab_panels, T);
     auto kern = forward_kernel_for(f64, h->cfg);
     CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -42,6 +42,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "table_eval.cuh"
 
 namespace {
 
@@ -54,7 +55,9 @@ __constant__ double c_gl_x[GL_N];   // 16-point Gauss-Legendre on [-1, 1]
 __constant__ double c_gl_w[GL_N];
 __constant__ double c_gl12_x[12];   // 12 points, for the tail
 __constant__ double c_gl12_w[12];
-__constant__ double c_dct[F64_NODES][F64_NODES];  // (2/n) cos(pi k (i + 1/2)/n), k = 0 halved
+// FP64 table: coefficients of a panel from the 10 node values of its build panel
+constexpr int F64_SPLIT = F64_FINE / F64_SUB, F64_COEF = 8;
+__constant__ double c_fit64[F64_SPLIT][F64_COEF][F64_NODES];
 // FP32 handles: 8 points, the 6 nodes' places and transform, the quadratic's 3 nodes
 __constant__ double c_gl8_x[8], c_gl8_w[8];
 __constant__ double c_cheb_t6[LITE_NODES], c_dct6[LITE_NODES][LITE_NODES];
@@ -656,7 +659,7 @@ table_nodes_kernel(const SampleParams *__restrict__ sp, double *__restrict__ scr
 // ---------------------------------------------------------------------------------
 template <bool LITE>
 __global__ void __launch_bounds__(K1_THREADS)
-table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scratch, double *__restrict__ tab64,
+table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scratch, float4 *__restrict__ tab64,
                    float4 *__restrict__ tab32, int max_oct) {
     extern __shared__ double sm[];
     __shared__ double s_part[2][K1_THREADS / 32];
@@ -671,14 +674,14 @@ table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scr
     const int M = p.n_oct * F64_SUB * NP;
     double *g1s = sm, *g2s = sm + M;  // [M] node values
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    double *t64 = tab64 + (size_t)b * TAB64_STRIDE;
+    float4 *t64 = tab64 + (size_t)b * TAB64_STRIDE;
     float4 *t32 = tab32 + (size_t)b * TAB32_STRIDE;
     const int at = blockIdx.y * K1_THREADS + tid, step = gridDim.y * K1_THREADS;
 
     if (p.status != SWIMMER_OK) {
         // keep the table finite so that a stray read cannot produce garbage
         if (!LITE)
-            for (int i = at; i < TAB64_STRIDE; i += step) t64[i] = 0.0;
+            for (int i = at; i < TAB64_STRIDE; i += step) t64[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         else
             for (int i = at; i < TAB32_STRIDE; i += step) t32[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         return;
@@ -787,15 +790,31 @@ table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scr
     __syncthreads();
 
     if (!LITE) {
-        // Chebyshev coefficients per FP64 panel: a_k = (2/n) sum_i g(t_i) T_k(t_i), a_0 halved
-        const int np64 = p.n_oct * F64_SUB;
-        for (int q = at; q < 2 * np64 * F64_NODES; q += step) {  // (a warp shares its row of c_dct)
-            const int f = q / (np64 * F64_NODES), rem = q % (np64 * F64_NODES);
-            const int panel = rem % np64, k = rem / np64;
-            const double *g = (f == 0 ? g1s : g2s) + panel * F64_NODES;
-            double s = 0.0;
-            for (int ii = 0; ii < F64_NODES; ++ii) s += g[ii] * c_dct[k][ii];
-            t64[(f * F64_PANELS_MAX + panel) * F64_NODES + k] = s;
+        // the panels' records (table_eval.cuh), four panels to a build panel
+        const int np = p.n_oct * F64_SUB;
+        for (int q = at; q < p.n_oct * F64_FINE; q += step) {  // (a warp shares its rows of c_fit64)
+            const int panel = q % np, part = q / np;
+            float4 *rec = t64 + F64_REC * (panel * F64_SPLIT + part);
+            const double *ga = g1s + panel * F64_NODES, *gb = g2s + panel * F64_NODES;
+            double ca[F64_COEF], cb[F64_COEF];
+#pragma unroll
+            for (int k = 0; k < F64_COEF; ++k) {
+                double x = 0.0, y = 0.0;
+                for (int i = 0; i < F64_NODES; ++i) {
+                    const double w = c_fit64[part][k][i];
+                    x = fma(w, ga[i], x);
+                    y = fma(w, gb[i], y);
+                }
+                ca[k] = x;
+                cb[k] = y;
+            }
+            *(double2 *)rec = make_double2(ca[0], cb[0]);
+#pragma unroll
+            for (int k = 1; k <= 5; ++k) {
+                const float ha = (float)ca[k], hb = (float)cb[k];
+                rec[k] = make_float4(ha, hb, (float)(ca[k] - (double)ha), (float)(cb[k] - (double)hb));
+            }
+            rec[6] = make_float4((float)ca[6], (float)cb[6], (float)ca[7], (float)cb[7]);
         }
         return;
     }
@@ -874,7 +893,7 @@ __global__ void set_sample_kernel(SampleParams *sp, double alpha, double delta, 
 // ---------------------------------------------------------------------------------
 __global__ void kernel_eval_kernel(int m, const double *__restrict__ r, double *__restrict__ g1,
                                    double *__restrict__ g2, const SampleParams *__restrict__ sp,
-                                   const double *__restrict__ tab64, const float4 *__restrict__ tab32,
+                                   const float4 *__restrict__ tab64, const float4 *__restrict__ tab32,
                                    int precision) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
@@ -882,24 +901,11 @@ __global__ void kernel_eval_kernel(int m, const double *__restrict__ r, double *
     double rr = r[i];
     if (precision == SWIMMER_FP64) {
         double u = 1.0 + rr * rr / (p.delta * p.delta);
-        unsigned long long bits = (unsigned long long)__double_as_longlong(u);
-        unsigned long long panel = (bits >> (52 - F64_SUB_LOG2)) - (1023ull << F64_SUB_LOG2);
-        if (!(u >= 1.0) || panel >= (unsigned long long)(p.n_oct * F64_SUB)) {
+        if (!(u >= 1.0) || !(u < ldexp(1.0, p.n_oct))) {
             g1[i] = g2[i] = nan("");
             return;
         }
-        double f = __longlong_as_double(0x3ff0000000000000LL | (long long)((bits << F64_SUB_LOG2) & 0x000fffffffffffffull)) - 1.0;
-        double t = 2.0 * f - 1.0;
-        for (int fn = 0; fn < 2; ++fn) {
-            const double *c = tab64 + (fn * F64_PANELS_MAX + panel) * F64_NODES;
-            double b1 = 0.0, b2 = 0.0;
-            for (int k = F64_DEG; k >= 1; --k) {
-                double b0 = 2.0 * t * b1 - b2 + c[k];
-                b2 = b1;
-                b1 = b0;
-            }
-            (fn == 0 ? g1 : g2)[i] = t * b1 - b2 + c[0];
-        }
+        kern_f64(tab64, p.n_oct * F64_FINE - 1, u, g1[i], g2[i]);
     } else {
         float inv_d2 = (float)(1.0 / (p.delta * p.delta));
         float r2 = (float)(rr * rr);
@@ -1004,6 +1010,19 @@ static void cheb_to_powers(double *c, int n) {
     }
     std::copy(out.begin(), out.end(), c);
 }
+// powers of t, t in [-1, 1] across [lo, hi], of f's polynomial through n Chebyshev nodes cut to
+// degree deg (its Chebyshev series, so that what is cut is small)
+void fit_powers(int n, int deg, double (*f)(double), double lo, double hi, double *c) {
+    std::vector<double> v(n);
+    for (int i = 0; i < n; ++i) v[i] = f(lo + 0.5 * (hi - lo) * (cos(PI * (i + 0.5) / n) + 1.0));
+    for (int k = 0; k <= deg; ++k) {
+        double s = 0.0;
+        for (int i = 0; i < n; ++i) s += v[i] * cos(PI * k * (i + 0.5) / n);
+        c[k] = s * (k == 0 ? 1.0 : 2.0) / n;
+    }
+    cheb_to_powers(c, deg + 1);
+}
+
 // powers of t = z_scale z + z_shift of f(1/z) on x in [lo, 1/inv_hi], degree deg
 template <class F>
 static void fit_inverse(double lo, double inv_hi, int deg, F f, double *c) {
@@ -1124,14 +1143,29 @@ int gl_init() {
     CUDA_TRY(cudaMemcpyToSymbol(c_i2p, pi1[1], sizeof(pi1[1])));
     CUDA_TRY(cudaMemcpyToSymbol(c_i0q, pi2[0], sizeof(pi2[0])));
     CUDA_TRY(cudaMemcpyToSymbol(c_i2q, pi2[1], sizeof(pi2[1])));
-    // table fits
-    double dct[F64_NODES][F64_NODES];
-    for (int ii = 0; ii < F64_NODES; ++ii) {
-        int i = F64_NODES - 1 - ii;  // ascending node ii is Chebyshev index i
-        for (int k = 0; k < F64_NODES; ++k)
-            dct[k][ii] = (2.0 / F64_NODES) * cos(PI * k * (i + 0.5) / F64_NODES) * (k == 0 ? 0.5 : 1.0);
-    }
-    CUDA_TRY(cudaMemcpyToSymbol(c_dct, dct, sizeof(dct)));
+    // FP64 table fits: the degree-9 polynomial through the 10 nodes, on a quarter of its panel,
+    // t = (tau + 2 part - 3) / 4, as a Chebyshev series in tau cut to degree 7 (what is cut is below
+    // 1e-17), in powers of tau
+    std::vector<double> fit(F64_SPLIT * F64_COEF * F64_NODES);
+    for (int part = 0; part < F64_SPLIT; ++part)
+        for (int ii = 0; ii < F64_NODES; ++ii) {
+            const int i = F64_NODES - 1 - ii;  // ascending node ii is Chebyshev index i
+            double v[F64_NODES], c[F64_NODES];
+            for (int j = 0; j < F64_NODES; ++j) {
+                const double t = 0.25 * (cos(PI * (j + 0.5) / F64_NODES) + 2.0 * part - 3.0);
+                v[j] = 1.0 / F64_NODES;
+                for (int k = 1; k < F64_NODES; ++k)
+                    v[j] += (2.0 / F64_NODES) * cos(PI * k * (i + 0.5) / F64_NODES) * cos(k * acos(t));
+            }
+            for (int k = 0; k < F64_NODES; ++k) {
+                c[k] = 0.0;
+                for (int j = 0; j < F64_NODES; ++j)
+                    c[k] += (k ? 2.0 : 1.0) / F64_NODES * v[j] * cos(PI * k * (j + 0.5) / F64_NODES);
+            }
+            cheb_to_powers(c, F64_COEF);
+            for (int k = 0; k < F64_COEF; ++k) fit[(part * F64_COEF + k) * F64_NODES + ii] = c[k];
+        }
+    CUDA_TRY(cudaMemcpyToSymbol(c_fit64, fit.data(), sizeof(double) * fit.size()));
     // FP32 handles
     double ik[NSER], ikk[2][NSER], hk[HARM];
     for (int k = 0; k < NSER; ++k) {
@@ -1201,7 +1235,7 @@ int launch_prepare(swimmer_handle *h, int B, const double *theta, const int *n_p
 }
 
 // the two table kernels on B samples whose scratch rows start at `scratch`
-static int table_kernels(int B, SampleParams *sp, double *scratch, double *tab64, float4 *tab32, bool lite, int oct,
+static int table_kernels(int B, SampleParams *sp, double *scratch, float4 *tab64, float4 *tab32, bool lite, int oct,
                          int sms, cudaStream_t s) {
     const int M = oct * F64_SUB * (lite ? LITE_NODES : F64_NODES);
     const dim3 ga(B, (M + K1A_THREADS - 1) / K1A_THREADS + 1);
@@ -1255,13 +1289,13 @@ int launch_kernel_eval(swimmer_handle *h, int m, const double *r, double *g1, do
 // ~0.2 MB until the process exits, and every call on a device shares them.
 namespace {
 __device__ __align__(256) double g_noalloc_scratch[K1_SCRATCH];
-__device__ __align__(256) double g_noalloc_tab64[TAB64_STRIDE];
+__device__ __align__(256) float4 g_noalloc_tab64[TAB64_STRIDE];
 __device__ __align__(256) float4 g_noalloc_tab32[TAB32_STRIDE];
 __device__ __align__(256) SampleParams g_noalloc_sp[1];
 
 struct NoallocPtrs {
-    double *scratch, *tab64;
-    float4 *tab32;
+    double *scratch;
+    float4 *tab64, *tab32;
     SampleParams *sp;
     bool ready;
 };
