@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(FLOW_THREADS) flow_kernel(int n, const double 
     for (int g0 = blockIdx.x * FLOW_THREADS; g0 < G; g0 += gridDim.x * FLOW_THREADS) {
         const int g = g0 + threadIdx.x;
         const double x = g < G ? grid[2 * (size_t)g] : 0.0, y = g < G ? grid[2 * (size_t)g + 1] : 0.0;
-        double vx = 0.0, vy = 0.0, pr = 0.0;
+        double ax = 0.0, ay = 0.0, vx = 0.0, vy = 0.0, pr = 0.0;  // sums of F g1, of (F . d) d h, of pressure
         for (int j0 = 0; j0 < n; j0 += FLOW_SOURCES) {
             const int m = min(FLOW_SOURCES, n - j0);
             if (!one_load || g0 == blockIdx.x * FLOW_THREADS) {
@@ -81,16 +81,18 @@ __global__ void __launch_bounds__(FLOW_THREADS) flow_kernel(int n, const double 
                     float2 qh, ql;
                     poly_f64(rec, th, tl, qh, ql);
                     const double g1 = c0.x + (widen(qh.x) + widen(ql.x)), w = fd * (c0.y + (widen(qh.y) + widen(ql.y)));
-                    vx = fma(w, dx, fma(-F.x, g1, vx));
-                    vy = fma(w, dy, fma(-F.y, g1, vy));
+                    ax = fma(F.x, g1, ax);
+                    ay = fma(F.y, g1, ay);
+                    vx = fma(w, dx, vx);
+                    vy = fma(w, dy, vy);
                 }
                 if (pres) pr = fma(fd, poly1_f64(ptab + PRES_REC * pan, th, tl), pr);
             }
         }
         if (g < G) {
             if (vel) {
-                vel[2 * (size_t)g] = vx * inv_mu;
-                vel[2 * (size_t)g + 1] = vy * inv_mu;
+                vel[2 * (size_t)g] = fma(vx, inv_d2, -ax) * inv_mu;
+                vel[2 * (size_t)g + 1] = fma(vy, inv_d2, -ay) * inv_mu;
             }
             if (pres) pres[g] = pr * inv_d2;
         }

@@ -1,21 +1,20 @@
-// K2: fused persistent forward model + log-likelihood, one CTA per sample at a time.
+// K2 in FP32 (forward64.cu: FP64): fused persistent forward model + log-likelihood, one CTA per
+// sample at a time.
 //
 // Per time step (Appendix, last paragraph; Sec. 2.1):
 //   A  segment vectors e_k = X_{k+1} - X_k and spring tension 2 K_T (|e_k|/ds - 1)/|e_k|
 //      (Eq. EFT read as Hookean springs).  The strain comes from |e|^2/ds^2 - 1 evaluated
-//      without cancellation (FP64 in the FP64 kernel; error-free FP32 transformations on
-//      the double-float positions in the FP32 kernel);
+//      without cancellation (error-free FP32 transformations on the double-float positions);
 //   B  (same pass) nonlinear curvature zeta_k (Eq. curva) from central differences,
 //      preferred curvature zeta^_k(t), and c_k d zeta_k / d X_{k-1,k,k+1} with
-//      c_k = 2 K_C ds (zeta - zeta^) (gradient of Eq. EFB).  The FP32 kernel takes the
+//      c_k = 2 K_C ds (zeta - zeta^) (gradient of Eq. EFB).  It takes the
 //      second differences from the double-float segments before rounding them, uses the
 //      hardware reciprocal square root, and forms zeta^_k = P_k cos(omega t) +
 //      Q_k sin(omega t) from per-run FP64 coefficients and an FP64 rotation of the phase;
 //   C  point forces F = -dE/dX (Eq. Fenergy) gathered from the stencils;
 //   D  Brinkmanlet pair sum (Eq. BrV) v_i = (1/mu) sum_j [-F_j g1 + (F_j . d) d g2],
 //      d = X_i - X_j, with g1, g2 from the per-sample shared-memory table (quadratic in
-//      G = 1 + f/64 in FP32; in FP64 degree 7, all but its leading term in pairs of floats).
-//      FP32: every unordered pair once.  g1, g2 and (F . d) d are even in d, so one table
+//      G = 1 + f/64).  Every unordered pair once.  g1, g2 and (F . d) d are even in d, so one table
 //      lookup serves v_i and v_j.  The points form blocks of 32; a warp takes a block pair
 //      (I, J) along diagonals: lane l holds target I*32 + l and meets source
 //      J*32 + (l + d) mod 32 at step d, so all lanes look up nearly the same table panel
@@ -31,10 +30,8 @@
 //      in a fixed order with TwoSum, so results do not depend on scheduling.  Launches
 //      whose shared memory holds an SM to one CTA of at most 512 threads use an
 //      instantiation compiled for 128 registers a thread.
-//      FP64: target i meets source i + d mod n at step d, the S threads of a target splitting
-//      the sources and combining with warp shuffles;
-//   E  forward Euler X += dt v: FP64 positions in the FP64 kernel, double-float (hi + lo
-//      FP32, about 48 significant bits) positions updated by TwoSum in the FP32 kernel;
+//   E  forward Euler X += dt v: double-float (hi + lo FP32, about 48 significant bits)
+//      positions updated by TwoSum;
 //      every obs_every steps the head point is compared with the observations and the
 //      squared residual accumulated in FP64 (Eq. fitness).
 // A run stops early, with status DIVERGED, when a velocity is not finite, a point moves
@@ -45,60 +42,11 @@
 #include <algorithm>
 #include <vector>
 
-#include "common.cuh"
-#include "table_eval.cuh"
+#include "forward_args.cuh"
 
 namespace {
 
 constexpr double PI = 3.14159265358979323846;
-
-struct FwdArgs {
-    int B;
-    const SampleParams *sp;
-    const int *order;
-    int *queue;
-    const float4 *tab64;
-    const float4 *tab32;
-    void *pq;  // [B][n_max] preferred-curvature coefficients (P_k, Q_k) per run (float2 or double2)
-    double mu, dt, kt, eta, omega;
-    double hr_over_ds, gap_over_ds, k_head_tens, k_head_c, k_neck_tens, k_neck_ang;  // head model
-    int obs_kind;
-    double swim_d;        // two swimmers: initial separation along y
-    double sigma_ratio;   // noise of the second observed component / the first
-    long long steps, obs_every;
-    const double *obs;
-    double sigma;
-    double *loglik;
-    double *head_traj;
-    double *speed;
-    double *final_state;  // optional [B][n_max][4]: (x, y, Fx, Fy) at the end of the run
-    int *status;
-    unsigned long long *work;      // [0] executed, [1] useful pair evaluations
-    unsigned long long *run_work;  // per-run pair evaluations (speculative launches)
-    int speculative;               // 1: the caller decides later which runs were useful
-    int n_max;
-    int threads;
-    int tab_panels;  // panels of the shared-memory table region (handle's octaves x panels/octave)
-    const unsigned *units;  // FP32 pair-unit lists (offsets header, then the lists)
-    int mode;               // FP32 pair units: 0 one-, 1 two-, 2 four-target
-};
-
-struct __align__(32) dbl4 {
-    double x, y, z, w;
-};
-
-template <bool F64>
-struct Types;
-template <>
-struct Types<false> {
-    typedef float R;
-    typedef float4 R4;
-};
-template <>
-struct Types<true> {
-    typedef double R;
-    typedef dbl4 R4;
-};
 
 // error-free transformations (Knuth TwoSum, Dekker Fast2Sum)
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
@@ -131,10 +79,6 @@ __device__ __forceinline__ void df_sub(const float *h, const float *l, int i, in
 struct RestF32 {
     float l0, l02_hi, l02_lo, inv_l02, k2;
 };
-struct RestF64 {
-    double l0, inv_l02, k2_l0;
-};
-
 __host__ __device__ inline RestF32 rest_f32(double l0, double k) {
     RestF32 r;
     r.l0 = (float)l0;
@@ -142,14 +86,6 @@ __host__ __device__ inline RestF32 rest_f32(double l0, double k) {
     r.l02_lo = (float)(l0 * l0 - (double)r.l02_hi);
     r.inv_l02 = (float)(1.0 / (l0 * l0));
     r.k2 = (float)(2.0 * k);
-    return r;
-}
-
-__host__ __device__ inline RestF64 rest_f64(double l0, double k) {
-    RestF64 r;
-    r.l0 = l0;
-    r.inv_l02 = 1.0 / (l0 * l0);
-    r.k2_l0 = 2.0 * k / l0;
     return r;
 }
 
@@ -177,24 +113,13 @@ __device__ __forceinline__ float spring_f32(const float *xh, const float *xl, co
     return __fdividef(r.k2 * strain, ell);
 }
 
-__device__ __forceinline__ double spring_f64(const double *sx, const double *sy, int i, int j, const RestF64 &r,
-                                             double &ex, double &ey, double &strain) {
-    ex = sx[j] - sx[i];
-    ey = sy[j] - sy[i];
-    const double s2 = fma(fma(ex, ex, ey * ey), r.inv_l02, -1.0);  // l^2/l0^2 - 1
-    const double rs = rsqrt(1.0 + s2);                             // l0/l
-    strain = s2 / fma(1.0 + s2, rs, 1.0);
-    return r.k2_l0 * strain * rs;
-}
-
-// table region in shared memory: FP32: float4 part A [P] then float2 part B [P] (24 bytes a
+// table region in shared memory: float4 part A [P] then float2 part B [P] (24 bytes a
 // panel), or with MERGED one 32-byte record per panel [P][2] float4, so that one address serves
 // both loads of a lookup (the 128-register instantiation, whose launches are held to one or two
 // CTAs per SM by other limits, so the larger table costs no occupancy there);
-// FP64: the panels' records (table_eval.cuh)
-template <bool F64, bool MERGED = false>
+template <bool MERGED = false>
 __host__ __device__ size_t table_bytes(int P) {
-    return F64 ? sizeof(float4) * P * F64_REC : (MERGED ? 2 * sizeof(float4) : sizeof(float4) + sizeof(float2)) * P;
+    return (MERGED ? 2 * sizeof(float4) : sizeof(float4) + sizeof(float2)) * P;
 }
 
 __host__ __device__ inline size_t align32(size_t b) { return (b + 31) & ~size_t(31); }
@@ -210,16 +135,12 @@ __host__ __device__ inline int pair_warps(int n_max, int threads) {
 }
 
 // Per-step state in shared memory.
-// FP64: positions sx, sy [n_max] (double); sources (x, y, Fx, Fy) [n_max]; tension vectors
-//   tx, ty [n_max]; six bending terms [6][n_max].
-// FP32: positions xh, xl, yh, yl [n_max]; sources per block of 32 points as two planes of
+// Positions xh, xl, yh, yl [n_max]; sources per block of 32 points as two planes of
 //   pair records ([nbm][2][32] float4, plane_a / plane_b); tension vectors and bending terms
 //   [8][n_max], which
 //   during the pair sum hold the per-warp partial velocities [pair warps][nbm * 32] (float2)
 //   instead, the region growing when those need more room.
-template <bool F64>
-__host__ __device__ size_t state_bytes(int n_max, int threads) {
-    if (F64) return align32(16 * (size_t)n_max) + 32 * (size_t)n_max + 8 * 8 * (size_t)n_max;
+__host__ __device__ inline size_t state_bytes(int n_max, int threads) {
     const size_t nbm = (n_max + 31) / 32;
     size_t forces = 32 * (size_t)n_max, part = 256 * nbm * (size_t)pair_warps(n_max, threads);
     // (the same bytes are the pair-unit assignment's scratch at the start of a sample)
@@ -230,10 +151,10 @@ __host__ __device__ size_t state_bytes(int n_max, int threads) {
 }
 
 // FP32: the sample's pair units (unit_pack), at most ceil(n_max/32)^2 ints after the table
-template <bool F64, bool MERGED = false>
+template <bool MERGED = false>
 __host__ __device__ size_t smem_bytes(int n_max, int P, int threads) {
     const size_t nbm = (n_max + 31) / 32;
-    return state_bytes<F64>(n_max, threads) + table_bytes<F64, MERGED>(P) + (F64 ? 0 : 4 * nbm * nbm);
+    return state_bytes(n_max, threads) + table_bytes<MERGED>(P) + 4 * nbm * nbm;
 }
 
 
@@ -393,24 +314,17 @@ __device__ __forceinline__ void assign_units(unsigned *units, int n_units, int n
     for (int u = 0; u < n_units; ++u) units[u] = tmp[u];
 }
 
-// observations computed by warp 0 after a step (head-centre velocities, two-swimmer
-// distances) rather than by the thread that updates the proximal point
-__device__ __forceinline__ bool vel_obs(const FwdArgs &a, int nh) {
-    return (a.obs_kind == SWIMMER_OBS_HEAD_VELOCITY || a.obs_kind == SWIMMER_OBS_PAIR_DISTANCES) && nh > 0;
-}
-
 // Mean of the head points (FP64 sums over one warp, fixed order); all lanes of warp 0 call
 // it, lane 0 gets the result.
-template <bool F64>
-__device__ __forceinline__ void head_centre(const double *sx, const double *sy, const float *xh, const float *xl,
+__device__ __forceinline__ void head_centre(const float *xh, const float *xl,
                                             const float *yh, const float *yl, int nf, int nh, int lane, double &cx,
                                             double &cy) {
     cx = 0.0;
     cy = 0.0;
     for (int m = lane; m < nh; m += 32) {
         const int k = nf + m;
-        cx += F64 ? sx[k] : (double)xh[k] + (double)xl[k];
-        cy += F64 ? sy[k] : (double)yh[k] + (double)yl[k];
+        cx += (double)xh[k] + (double)xl[k];
+        cy += (double)yh[k] + (double)yl[k];
     }
     for (int o = 16; o >= 1; o >>= 1) {
         cx += __shfl_xor_sync(0xffffffffu, cx, o);
@@ -425,43 +339,40 @@ __device__ __forceinline__ void head_centre(const double *sx, const double *sy, 
 // for at most 512 threads and one CTA per SM (up to 128 registers a thread), for launches
 // whose shared memory already holds them to that few threads per SM (large N): the pair
 // loop then keeps more loads in flight.
-template <bool F64, int MODEL, bool BIG = false>
+template <int MODEL, bool BIG = false>
 __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a) {
     constexpr bool HEAD = MODEL >= 1, TWO = MODEL == 2;
-    constexpr bool MERGED = !F64 && BIG;  // the FP32 table as 32-byte records (see table_bytes)
-    typedef typename Types<F64>::R R;
-    typedef typename Types<F64>::R4 R4;
+    constexpr bool MERGED = BIG;  // the FP32 table as 32-byte records (see table_bytes)
+    typedef float R;
+    typedef float4 R4;
     extern __shared__ __align__(32) unsigned char smraw[];
     const int n_max = a.n_max;
-    // positions: FP64 kernel sx, sy (double); FP32 kernel xh, xl, yh, yl (float)
-    double *sx = (double *)smraw;
-    double *sy = sx + n_max;
+    // positions as double-floats
     float *xh = (float *)smraw, *xl = xh + n_max, *yh = xl + n_max, *yl = yh + n_max;
     const int nbm = (n_max + 31) >> 5;
-    R4 *src = (R4 *)(smraw + align32(16 * (size_t)n_max));  // FP64 [n_max]; FP32 [nbm][64]
-    R *tvx = (R *)(src + (F64 ? n_max : 64 * nbm));    // tension vectors, then bending
+    R4 *src = (R4 *)(smraw + align32(16 * (size_t)n_max));  // [nbm][64]
+    R *tvx = (R *)(src + 64 * nbm);  // tension vectors, then bending
     R *tvy = tvx + n_max;
     R *bend = tvy + n_max;  // [6][n_max]
     float2 *part = (float2 *)tvx;  // FP32 pair sum: per-warp partial velocities
-    unsigned char *tabraw = smraw + state_bytes<F64>(n_max, blockDim.x);
+    unsigned char *tabraw = smraw + state_bytes(n_max, blockDim.x);
     __shared__ int s_work;
     // the sample's model constants: [0, 18) the springs (flagellum segment, head membrane,
     // diametral, neck A (end to H(pi +- dth)), neck B (next-to-end to H(pi +- dth)), neck
-    // gap (end to H(pi))) as RestF64 or RestF32 records; then 1/(2 ds_H), 1/ds_H^2, 1/H_r,
+    // gap (end to H(pi))) as RestF32 records; then 1/(2 ds_H), 1/ds_H^2, 1/H_r,
     // 2 K_HC ds_H, 2 K_NA; [23, 25) the head centre at the previous observation
     __shared__ double s_model[26];
     // FP32 kernel: the sample's single-precision constants (see below)
     enum { F_DS, F_INV2DS, F_INVDS2, F_KC2DS, F_INVDELTA, F_DTMU, F_COUNT };
-    __shared__ float s_f32[F64 ? 1 : 16];
+    __shared__ float s_f32[16];
     // FP32 kernel: (cos, sin)(omega t) of the current step, and the FP64 rotation state
     // (cos, sin)(omega step dt), (cos, sin)(omega dt) that thread 0 advances once per step
     __shared__ float s_rot[2];
-    __shared__ double s_rot64[F64 ? 64 : 4];  // FP64 kernel: (cos, sin)(omega t) of 32 steps
+    __shared__ double s_rot64[4];
     // FP32 pair sum: warp w processes units [s_wstart[w], s_wstart[w + 1]) of the sample's list
-    __shared__ int s_wstart[F64 ? 1 : 33];
+    __shared__ int s_wstart[33];
     static_assert(F_COUNT <= 16, "s_f32 holds 16 constants");
     const RestF32 *rest32 = (const RestF32 *)s_model;
-    const RestF64 *rest64 = (const RestF64 *)s_model;
     enum { M_I2H = 18, M_IH2, M_IHR, M_KHC, M_KANG, M_CX, M_CY };
 
     const int tid = threadIdx.x, T = blockDim.x;
@@ -492,38 +403,31 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
         }
         // ---- table into shared memory
         const int P = a.tab_panels;
-        const int npan = min(P, p.n_oct * (F64 ? F64_FINE : F32_SUB));
-        if (F64) {
-            const float4 *g = a.tab64 + (size_t)b * TAB64_STRIDE;
-            float4 *t = (float4 *)tabraw;
-            for (int i = tid; i < npan * F64_REC; i += T) t[i] = g[i];
-        } else {
-            const float4 *g = a.tab32 + (size_t)b * TAB32_STRIDE;
-            const float2 *gb = (const float2 *)(g + F32_PANELS_MAX);
-            float4 *t = (float4 *)tabraw;
-            float2 *tb = (float2 *)(t + P);
-            for (int i = tid; i < npan; i += T) {
-                if (MERGED) {
-                    t[2 * i] = g[i];
-                    t[2 * i + 1] = make_float4(gb[i].x, gb[i].y, 0.f, 0.f);
-                } else {
-                    t[i] = g[i];
-                    tb[i] = gb[i];
-                }
+        const int npan = min(P, p.n_oct * F32_SUB);
+        const float4 *g = a.tab32 + (size_t)b * TAB32_STRIDE;
+        const float2 *gb = (const float2 *)(g + F32_PANELS_MAX);
+        float4 *t = (float4 *)tabraw;
+        float2 *tb = (float2 *)(t + P);
+        for (int i = tid; i < npan; i += T) {
+            if (MERGED) {
+                t[2 * i] = g[i];
+                t[2 * i + 1] = make_float4(gb[i].x, gb[i].y, 0.f, 0.f);
+            } else {
+                t[i] = g[i];
+                tb[i] = gb[i];
             }
-            // the sample's pair units, from the handle's list for its block count
-            const int nbs = (n + 31) >> 5;
-            const unsigned *hdr = a.units + a.mode * (UNIT_NB_MAX + 1);
-            const unsigned *ul = a.units + UNIT_HDR + hdr[nbs - 1];
-            unsigned *units = (unsigned *)(tabraw + table_bytes<F64, MERGED>(P));
-            for (int un = tid; un < (int)(hdr[nbs] - hdr[nbs - 1]); un += T) units[un] = ul[un];
         }
+        // the sample's pair units, from the handle's list for its block count
+        const int nbs = (n + 31) >> 5;
+        const unsigned *hdr = a.units + a.mode * (UNIT_NB_MAX + 1);
+        const unsigned *ul = a.units + UNIT_HDR + hdr[nbs - 1];
+        unsigned *units = (unsigned *)(tabraw + table_bytes<MERGED>(P));
+        for (int un = tid; un < (int)(hdr[nbs] - hdr[nbs - 1]); un += T) units[un] = ul[un];
         // ---- initial straight filament X_k = (k ds, 0), stored relative to (L/2, 0); the
         //      head circle's centre H_r + dN to the right of the proximal point, head point m
         //      at angle 2 pi m / N_H (Appendix)
         const double ds = p.ds, L = p.length;
         const double xref = 0.5 * L;
-        {
         const double hr = a.hr_over_ds * ds, gap = a.gap_over_ds * ds;
         const double dth = nh ? 2.0 * PI / nh : 0.0, dsh = hr * dth;
         for (int k = tid; k < n; k += T) {
@@ -540,17 +444,12 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 y0 = hr * sn;
             }
             if (sw) y0 += a.swim_d;
-            if (F64) {
-                sx[k] = x0;
-                sy[k] = y0;
-            } else {
-                float h = (float)x0;
-                xh[k] = h;
-                xl[k] = (float)(x0 - (double)h);
-                h = (float)y0;
-                yh[k] = h;
-                yl[k] = (float)(y0 - (double)h);
-            }
+            float h = (float)x0;
+            xh[k] = h;
+            xl[k] = (float)(x0 - (double)h);
+            h = (float)y0;
+            yh[k] = h;
+            yl[k] = (float)(y0 - (double)h);
         }
         if (tid == 0) {
             const double c1 = hr * (1.0 - cos(dth)), s1 = hr * sin(dth);
@@ -559,10 +458,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
             const double kk[6] = {a.kt, a.k_head_tens, a.k_head_tens, a.k_neck_tens, a.k_neck_tens, a.k_neck_tens};
             for (int q = 0; q < 6; ++q) {
                 const double lq = l0[q] > 0.0 ? l0[q] : 1.0;  // unused without a head
-                if (F64)
-                    ((RestF64 *)s_model)[q] = rest_f64(lq, kk[q]);
-                else
-                    ((RestF32 *)s_model)[q] = rest_f32(lq, kk[q]);
+                ((RestF32 *)s_model)[q] = rest_f32(lq, kk[q]);
             }
             s_model[M_I2H] = nh ? 0.5 / dsh : 0.0;
             s_model[M_IH2] = nh ? 1.0 / (dsh * dsh) : 0.0;
@@ -570,25 +466,23 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
             s_model[M_KHC] = 2.0 * a.k_head_c * dsh;
             s_model[M_KANG] = 2.0 * a.k_neck_ang;
         }
+        // pad the last block with force-free sources at the origin
+        const int npad = ((n + 31) >> 5) << 5;
+        for (int k = n + tid; k < npad; k += T) {
+            src[plane_a(k)] = R4{0, 0, 0, 0};
+            src[plane_b(k)] = R4{0, 0, 0, 0};
         }
-        if (!F64) {  // pad the last block with force-free sources at the origin
-            const int npad = ((n + 31) >> 5) << 5;
-            for (int k = n + tid; k < npad; k += T) {
-                src[plane_a(k)] = R4{0, 0, 0, 0};
-                src[plane_b(k)] = R4{0, 0, 0, 0};
-            }
-            if (n < npad && tid == 0) {  // the last point's entries pair it with the first pad
-                const int kp = plane_prev(n);
-                src[plane_a(kp)].y = 0;
-                src[plane_a(kp)].w = 0;
-                src[plane_b(kp)].y = 0;
-                src[plane_b(kp)].w = 0;
-            }
+        if (n < npad && tid == 0) {  // the last point's entries pair it with the first pad
+            const int kp = plane_prev(n);
+            src[plane_a(kp)].y = 0;
+            src[plane_a(kp)].w = 0;
+            src[plane_b(kp)].y = 0;
+            src[plane_b(kp)].w = 0;
         }
         // FP32 kernel: the sample's single-precision constants, made once here in FP64 and read
         // from shared memory in the step loop (where, short of registers, the compiler would
         // otherwise recompute them from the FP64 parameters every step)
-        if (!F64 && tid == 0) {
+        if (tid == 0) {
             s_f32[F_DS] = (float)ds;
             s_f32[F_INV2DS] = (float)(0.5 / ds);
             s_f32[F_INVDS2] = (float)(1.0 / (ds * ds));
@@ -605,63 +499,47 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
             s_rot[0] = 1.f;
             s_rot[1] = 0.f;
         }
-        {
-            // the preferred curvature of flagellum point k (Appendix: y^ = a (1 - s/L)
-            // sin(eta s - omega t), zeta^ = d^2 y^/ds^2) split as
-            // zeta^_k(t) = P_k cos(omega t) + Q_k sin(omega t), made in FP64 once per run
-            const size_t row = (size_t)b * n_max;
-            for (int k = tid; k < nf; k += T) {
-                const double sk = k * ds;
-                double sn, cs;
-                sincos(a.eta * sk, &sn, &cs);
-                const double c1 = 2.0 * a.eta / L, c2 = (1.0 - sk / L) * a.eta * a.eta;
-                const double pk = -p.amp * (c1 * cs + c2 * sn), qk = -p.amp * (c1 * sn - c2 * cs);
-                if (F64)
-                    ((double2 *)a.pq)[row + k] = make_double2(pk, qk);
-                else
-                    ((float2 *)a.pq)[row + k] = make_float2((float)pk, (float)qk);
-            }
+        // the preferred curvature of flagellum point k (Appendix: y^ = a (1 - s/L)
+        // sin(eta s - omega t), zeta^ = d^2 y^/ds^2) split as
+        // zeta^_k(t) = P_k cos(omega t) + Q_k sin(omega t), made in FP64 once per run
+        const size_t row = (size_t)b * n_max;
+        for (int k = tid; k < nf; k += T) {
+            const double sk = k * ds;
+            double sn, cs;
+            sincos(a.eta * sk, &sn, &cs);
+            const double c1 = 2.0 * a.eta / L, c2 = (1.0 - sk / L) * a.eta * a.eta;
+            const double pk = -p.amp * (c1 * cs + c2 * sn), qk = -p.amp * (c1 * sn - c2 * cs);
+            a.pq[row + k] = make_float2((float)pk, (float)qk);
         }
-        const double dt_mu = a.dt / a.mu;
-        // FP64 pair sum: thread -> (target, source split of S lanes)
-        int S = 1;
-        while (S < 32 && 2 * S * n <= T) S <<= 1;
-        const int slot = tid / S, split = tid % S;
-        const int tgt = slot;  // one target per slot
-        const bool owner = (split == 0) && (tgt < n);
         // FP32 pair sum: the sample's units of 16 steps over the pair warps
         const unsigned *uhdr = a.units + a.mode * (UNIT_NB_MAX + 1);
-        const int nb = (n + 31) >> 5, n_units = F64 ? 0 : (int)(uhdr[nb] - uhdr[nb - 1]);
-        const int n_pw = F64 ? 0 : min(pair_warps(n_max, T), (int)(uhdr[nbm] - uhdr[nbm - 1]));
+        const int nb = (n + 31) >> 5, n_units = (int)(uhdr[nb] - uhdr[nb - 1]);
+        const int n_pw = min(pair_warps(n_max, T), (int)(uhdr[nbm] - uhdr[nbm - 1]));
         // the thread that keeps the log-likelihood: thread 0 for head-centre velocities (one
         // warp reduces the head after each observation step), else the one that updates the
         // proximal flagellum point nf - 1 (the observed point)
-        const bool head_thread = vel_obs(a, nh) ? tid == 0 : F64 ? (owner && tgt == nf - 1) : (tid == (nf - 1) % T);
+        const bool head_thread = vel_obs(a, nh) ? tid == 0 : tid == (nf - 1) % T;
         double J = 0.0;
         int status = SWIMMER_OK;
         long long steps_done = a.steps;
         __syncthreads();
-        if (!F64 && tid == 0)
-            assign_units((unsigned *)(tabraw + table_bytes<F64, MERGED>(P)), n_units, n_pw, (unsigned *)part, s_wstart);
+        if (tid == 0)
+            assign_units((unsigned *)(tabraw + table_bytes<MERGED>(P)), n_units, n_pw, (unsigned *)part, s_wstart);
         __syncthreads();
-        const R r_inv2ds = F64 ? (R)(0.5 / ds) : (R)s_f32[F_INV2DS];
-        const R r_invds2 = F64 ? (R)(1.0 / (ds * ds)) : (R)s_f32[F_INVDS2];
-        const R kc2ds = F64 ? (R)(2.0 * p.kc * ds) : (R)s_f32[F_KC2DS];
-        const R inv_d2 = (R)(1.0 / (p.delta * p.delta));
+        const R r_inv2ds = (R)s_f32[F_INV2DS];
+        const R r_invds2 = (R)s_f32[F_INVDS2];
+        const R kc2ds = (R)s_f32[F_KC2DS];
         if (vel_obs(a, nh) && tid < 32) {  // head centre at the previous observation
             double cx, cy;
-            head_centre<F64>(sx, sy, xh, xl, yh, yl, nf, nh, lane, cx, cy);
+            head_centre(xh, xl, yh, yl, nf, nh, lane, cx, cy);
             if (tid == 0) {
                 s_model[M_CX] = cx;
                 s_model[M_CY] = cy;
             }
         }
-        float g10 = 0.f;  // FP32: -g1 at r = 0 (self term)
-        if (!F64) {
-            float g2unused;
-            kern_f32<MERGED>((const float4 *)tabraw, (const float2 *)((const float4 *)tabraw + P), npan - 1, 1.0f,
-                             g10, g2unused);
-        }
+        float g10 = 0.f, g2unused;  // -g1 at r = 0 (self term)
+        kern_f32<MERGED>((const float4 *)tabraw, (const float2 *)((const float4 *)tabraw + P), npan - 1, 1.0f,
+                         g10, g2unused);
 
         // with a final state requested, one more pass of the force phases at t = steps dt
         const long long last = a.steps + (a.final_state ? 1 : 0);
@@ -671,10 +549,6 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
         const int obs_every = (int)min(a.obs_every, (long long)INT_MAX);  // > steps: no observation
         int obs_left = obs_every, obs_idx = 0;
         for (int step = 0; step < (int)last; ++step) {
-            if (F64 && (step & 31) == 0) {  // (the last reads of s_rot64 lie before a barrier)
-                if (tid >= T - 32) sincos(a.omega * ((double)(step + lane) * a.dt), &s_rot64[2 * lane + 1], &s_rot64[2 * lane]);
-                __syncthreads();
-            }
             const bool obs_step = --obs_left == 0;
             int bad = 0;
             // ---- A+B: segments, tension, curvature stencils, relative positions.  Thread k
@@ -691,77 +565,52 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 const bool center = hd || (kl >= 1 && kl + 1 < nf);
                 R qx, qy, epx = 0, epy = 0, emx = 0, emy = 0, tk = 0;
                 float d2x = 0.f, d2y = 0.f;  // FP32: e_k - e_{k-1} from the double-float segments
-                if (F64) {
-                    if (next >= 0) {
-                        double ex, ey, strain;
-                        tk = (R)spring_f64(sx, sy, k, next, rest64[hd ? 1 : 0], ex, ey, strain);
-                        epx = (R)ex;
-                        epy = (R)ey;
-                        if (!(fabs(strain) <= STRETCH_MAX)) bad = 1;
-                    }
-                    if (center) {
-                        emx = (R)(sx[k] - sx[prev]);
-                        emy = (R)(sy[k] - sy[prev]);
-                    }
-                    qx = (R)sx[k];
-                    qy = (R)sy[k];
-                } else {
-                    float epxl = 0.f, epyl = 0.f;
-                    if (next >= 0) {
-                        float strain, ex, ey;
-                        tk = (R)spring_f32(xh, xl, yh, yl, k, next, rest32[hd ? 1 : 0], ex, ey, epxl, epyl, strain);
-                        epx = (R)ex;
-                        epy = (R)ey;
-                        if (!(fabsf(strain) <= (float)STRETCH_MAX)) bad = 1;
-                    }
-                    if (center) {
-                        // e_{k-1} as a double-float (s, lo); the second difference e_k - e_{k-1}
-                        // subtracts the high parts first (neighbouring segments are close, so
-                        // that difference is exact) and then the low parts: rounding the
-                        // segments to FP32 before subtracting would leave it an error of
-                        // about 6e-8 ds, amplified by 1/ds^2 in the curvature
-                        float s, e, lo;
-                        two_sum(xh[k], -xh[prev], s, e);
-                        lo = e + (xl[k] - xl[prev]);
-                        emx = (R)(s + lo);
-                        d2x = (epx - s) + (epxl - lo);
-                        two_sum(yh[k], -yh[prev], s, e);
-                        lo = e + (yl[k] - yl[prev]);
-                        emy = (R)(s + lo);
-                        d2y = (epy - s) + (epyl - lo);
-                    }
-                    // the pair sum measures separations in units of delta
-                    qx = (R)((xh[k] + xl[k]) * s_f32[F_INVDELTA]);
-                    qy = (R)((yh[k] + yl[k]) * s_f32[F_INVDELTA]);
+                float epxl = 0.f, epyl = 0.f;
+                if (next >= 0) {
+                    float strain, ex, ey;
+                    tk = (R)spring_f32(xh, xl, yh, yl, k, next, rest32[hd ? 1 : 0], ex, ey, epxl, epyl, strain);
+                    epx = (R)ex;
+                    epy = (R)ey;
+                    if (!(fabsf(strain) <= (float)STRETCH_MAX)) bad = 1;
                 }
+                if (center) {
+                    // e_{k-1} as a double-float (s, lo); the second difference e_k - e_{k-1}
+                    // subtracts the high parts first (neighbouring segments are close, so
+                    // that difference is exact) and then the low parts: rounding the
+                    // segments to FP32 before subtracting would leave it an error of
+                    // about 6e-8 ds, amplified by 1/ds^2 in the curvature
+                    float s, e, lo;
+                    two_sum(xh[k], -xh[prev], s, e);
+                    lo = e + (xl[k] - xl[prev]);
+                    emx = (R)(s + lo);
+                    d2x = (epx - s) + (epxl - lo);
+                    two_sum(yh[k], -yh[prev], s, e);
+                    lo = e + (yl[k] - yl[prev]);
+                    emy = (R)(s + lo);
+                    d2y = (epy - s) + (epyl - lo);
+                }
+                // the pair sum measures separations in units of delta
+                qx = (R)((xh[k] + xl[k]) * s_f32[F_INVDELTA]);
+                qy = (R)((yh[k] + yl[k]) * s_f32[F_INVDELTA]);
                 if (next >= 0) {  // tension force vector of segment (k, next)
                     tvx[k] = tk * epx;
                     tvy[k] = tk * epy;
                 }
-                if (F64) {
-                    src[k].x = qx;
-                    src[k].y = qy;
-                } else {  // plane A: own entry, and the previous entry's second half
-                    const int ka = plane_a(k), kp = plane_a(plane_prev(k));
-                    src[ka].x = qx;
-                    src[ka].z = qy;
-                    src[kp].y = qx;
-                    src[kp].w = qy;
-                }
+                const int ka = plane_a(k), kp = plane_a(plane_prev(k));
+                src[ka].x = qx;
+                src[ka].z = qy;
+                src[kp].y = qx;
+                src[kp].w = qy;
                 if (center) {
                     const R i2h = hd ? (R)s_model[M_I2H] : r_inv2ds, ih2 = hd ? (R)s_model[M_IH2] : r_invds2;
                     R A = (emx + epx) * i2h, Bv = (emy + epy) * i2h;
-                    R C = (F64 ? epx - emx : (R)d2x) * ih2, D = (F64 ? epy - emy : (R)d2y) * ih2;
+                    R C = (R)d2x * ih2, D = (R)d2y * ih2;
                     R S2 = A * A + Bv * Bv;
                     R rs;
-                    if (F64) {
-                        rs = (R)rsqrt((double)S2);
-                    } else {
-                        // the hardware estimate plus one Newton step: its ~2 ulp error would
-                        // otherwise enter zeta and the stencils, which multiply it by 1/ds^2
-                        const float r0 = rsqrtf((float)S2);
-                        rs = (R)fmaf(r0 * 0.5f, fmaf(-(float)S2 * r0, r0, 1.0f), r0);
-                    }
+                    // the hardware estimate plus one Newton step: its ~2 ulp error would
+                    // otherwise enter zeta and the stencils, which multiply it by 1/ds^2
+                    const float r0 = rsqrtf((float)S2);
+                    rs = (R)fmaf(r0 * 0.5f, fmaf(-(float)S2 * r0, r0, 1.0f), r0);
                     R S15 = rs * rs * rs;
                     R S25 = S15 * rs * rs;
                     R cross = A * D - Bv * C;
@@ -770,16 +619,10 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                     if (hd) {
                         zhat = (R)s_model[M_IHR];  // preferred head curvature 1/H_r
                     } else {
-                        // zeta^_k(t) = P_k cos(omega t) + Q_k sin(omega t), P and Q made in FP64 for
-                        // the run.  FP64: the cosines and sines of 32 steps at a time, a lane each;
-                        // FP32: rotated in FP64 once per step
-                        if (F64) {
-                            const double2 c = ((const double2 *)a.pq)[(size_t)b * n_max + kl];
-                            zhat = (R)fma(c.x, s_rot64[2 * (step & 31)], c.y * s_rot64[2 * (step & 31) + 1]);
-                        } else {
-                            const float2 c = ((const float2 *)a.pq)[(size_t)b * n_max + kl];
-                            zhat = (R)fmaf(c.x, s_rot[0], c.y * s_rot[1]);
-                        }
+                        // zeta^_k(t) = P_k cos(omega t) + Q_k sin(omega t) (made in FP64 for the
+                        // run); (cos, sin)(omega t) is advanced in FP64 once per step
+                        const float2 c = a.pq[(size_t)b * n_max + kl];
+                        zhat = (R)fmaf(c.x, s_rot[0], c.y * s_rot[1]);
                     }
                     R ck = (hd ? (R)s_model[M_KHC] : kc2ds) * (zeta - zhat);
                     R za = D * S15 - (R)3 * A * cross * S25;
@@ -796,7 +639,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
             __syncthreads();
             // (cos, sin)(omega t) of the next step, rotated in FP64 by the last thread, which
             // has the fewest points here (this step's values were read before the barrier)
-            if (!F64 && tid == T - 1) {
+            if (tid == T - 1) {
                 const double c = s_rot64[0], sn = s_rot64[1], wc = s_rot64[2], ws = s_rot64[3];
                 const double nc = fma(c, wc, -sn * ws), ns = fma(sn, wc, c * ws);
                 s_rot64[0] = nc;
@@ -858,42 +701,26 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                         }
                         if (j < 0) continue;
                         j += base;
-                        if (F64) {
-                            const RestF64 &r = rest64[2 + kind];
-                            double ex, ey, strain;
-                            double t = spring_f64(sx, sy, k, j, r, ex, ey, strain);
-                            fx += (R)(t * ex);
-                            fy += (R)(t * ey);
-                            if (!(fabs(strain) <= STRETCH_MAX)) bad = 1;
-                        } else {
-                            const RestF32 &r = rest32[2 + kind];
-                            float ex, ey, exl, eyl, strain;
-                            float t = spring_f32(xh, xl, yh, yl, k, j, r, ex, ey, exl, eyl, strain);
-                            fx += (R)(t * ex);
-                            fy += (R)(t * ey);
-                            if (!(fabsf(strain) <= (float)STRETCH_MAX)) bad = 1;
-                        }
+                        const RestF32 &r = rest32[2 + kind];
+                        float ex, ey, exl, eyl, strain;
+                        float t = spring_f32(xh, xl, yh, yl, k, j, r, ex, ey, exl, eyl, strain);
+                        fx += (R)(t * ex);
+                        fy += (R)(t * ey);
+                        if (!(fabsf(strain) <= (float)STRETCH_MAX)) bad = 1;
                     }
                     // neck angle E = K (z1 . z2)^2, z1 = H(pi) - X_{nf-1}, z2 = H(pi+dth) - H(pi-dth)
                     const int ihp = base + nf + h2, iplus = ihp + 1, iminus = ihp - 1, iend = base + nf - 1;
                     if (k == ihp || k == iplus || k == iminus || k == iend) {
                         R z1x, z1y, z2x, z2y;
-                        if (F64) {
-                            z1x = (R)(sx[ihp] - sx[iend]);
-                            z1y = (R)(sy[ihp] - sy[iend]);
-                            z2x = (R)(sx[iplus] - sx[iminus]);
-                            z2y = (R)(sy[iplus] - sy[iminus]);
-                        } else {
-                            float h, l;
-                            df_sub(xh, xl, iend, ihp, h, l);
-                            z1x = (R)(h + l);
-                            df_sub(yh, yl, iend, ihp, h, l);
-                            z1y = (R)(h + l);
-                            df_sub(xh, xl, iminus, iplus, h, l);
-                            z2x = (R)(h + l);
-                            df_sub(yh, yl, iminus, iplus, h, l);
-                            z2y = (R)(h + l);
-                        }
+                        float h, l;
+                        df_sub(xh, xl, iend, ihp, h, l);
+                        z1x = (R)(h + l);
+                        df_sub(yh, yl, iend, ihp, h, l);
+                        z1y = (R)(h + l);
+                        df_sub(xh, xl, iminus, iplus, h, l);
+                        z2x = (R)(h + l);
+                        df_sub(yh, yl, iminus, iplus, h, l);
+                        z2y = (R)(h + l);
                         const R w = (R)s_model[M_KANG] * (z1x * z2x + z1y * z2y);
                         if (k == ihp) {
                             fx -= w * z2x;
@@ -910,61 +737,25 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                         }
                     }
                 }
-                if (F64) {
-                    src[k].z = fx;
-                    src[k].w = fy;
-                } else {  // plane B
-                    const int kb = plane_b(k), kp = plane_b(plane_prev(k));
-                    src[kb].x = fx;
-                    src[kb].z = fy;
-                    src[kp].y = fx;
-                    src[kp].w = fy;
-                }
+                const int kb = plane_b(k), kp = plane_b(plane_prev(k));
+                src[kb].x = fx;
+                src[kb].z = fy;
+                src[kp].y = fx;
+                src[kp].w = fy;
             }
             __syncthreads();
             if (step == a.steps) {  // final state: positions and the forces there
                 for (int k = tid; k < n; k += T) {
                     double *o = a.final_state + ((size_t)b * n_max + k) * 4;
-                    o[0] = (F64 ? sx[k] : (double)xh[k] + (double)xl[k]) + xref;
-                    o[1] = F64 ? sy[k] : (double)yh[k] + (double)yl[k];
-                    o[2] = F64 ? (double)src[k].z : (double)src[plane_b(k)].x;
-                    o[3] = F64 ? (double)src[k].w : (double)src[plane_b(k)].z;
+                    o[0] = ((double)xh[k] + (double)xl[k]) + xref;
+                    o[1] = (double)yh[k] + (double)yl[k];
+                    o[2] = (double)src[plane_b(k)].x;
+                    o[3] = (double)src[plane_b(k)].z;
                 }
                 break;
             }
             // ---- D: pair sum
-            double vxd = 0.0, vyd = 0.0;
-            if (F64) {
-                // FP64: target tgt meets source tgt + d at step d (d = split, split + S, ...)
-                if (tgt < n) {
-                    const R4 me = src[tgt];
-                    const double xi = (double)me.x, yi = (double)me.y;
-                    const float4 *tab = (const float4 *)tabraw;
-                    double vx = 0.0, vy = 0.0;
-                    int j = tgt + split;
-                    if (j >= n) j -= n;
-                    for (int d = split; d < n; d += S) {
-                        const R4 q = src[j];
-                        j += S;
-                        if (j >= n) j -= n;
-                        double dx = xi - (double)q.x, dy = yi - (double)q.y;
-                        double u = fma(fma(dx, dx, dy * dy), (double)inv_d2, 1.0);
-                        double g1, g2;
-                        kern_f64(tab, npan - 1, u, g1, g2);
-                        double fd = fma((double)q.z, dx, (double)q.w * dy);
-                        double wv = fd * g2;
-                        vx = fma(wv, dx, fma(-(double)q.z, g1, vx));
-                        vy = fma(wv, dy, fma(-(double)q.w, g1, vy));
-                    }
-                    vxd = vx;
-                    vyd = vy;
-                }
-                // combine the S source splits (lanes of one warp)
-                for (int o = S >> 1; o >= 1; o >>= 1) {
-                    vxd += __shfl_xor_sync(0xffffffffu, vxd, o);
-                    vyd += __shfl_xor_sync(0xffffffffu, vyd, o);
-                }
-            } else if ((tid >> 5) < n_pw) {
+            if ((tid >> 5) < n_pw) {
                 // FP32: each unordered pair {i, j} once.  g1(r) and g2(r) are even in
                 // d = X_i - X_j and (F . d) d is even too, so one table lookup gives both
                 // v_i += -F_j g1 + (F_j . d) d g2 and v_j += -F_i g1 + (F_i . d) d g2.
@@ -985,7 +776,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 const int warp = tid >> 5;
                 float2 *mypart = part + warp * (nb << 5);
                 for (int k = lane; k < (nb << 5); k += 32) mypart[k] = make_float2(0.f, 0.f);
-                const unsigned *units = (const unsigned *)(tabraw + table_bytes<F64, MERGED>(P));
+                const unsigned *units = (const unsigned *)(tabraw + table_bytes<MERGED>(P));
                 for (int un = s_wstart[warp]; un < s_wstart[warp + 1]; ++un) {
                     const unsigned pk = units[un];
                     const int I = pk & 31, Jb = (pk >> 5) & 31, code = (pk >> 25) & 3, kind = (pk >> 27) & 3;
@@ -1006,41 +797,34 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                     }
                 }
             }
-            if (!F64) __syncthreads();
+            __syncthreads();
             // ---- E: Euler step, divergence, observations
-            for (int k = F64 ? (owner ? tgt : n) : tid; k < n; k += F64 ? n : T) {
-                if (F64) {
-                    double dx = vxd * dt_mu, dy = vyd * dt_mu;  // displacement this step
-                    if (!isfinite(dx) || !isfinite(dy) || fmax(fabs(dx), fabs(dy)) > ds) bad = 1;
-                    sx[k] += dx;
-                    sy[k] += dy;
-                } else {
-                    // v_k = self term + the pair warps' partial sums, compensated
-                    const float4 fk = ((const float4 *)src)[plane_b(k)];  // (Fx, ., Fy, .)
-                    float hx = fk.x * g10, lx = 0.f, hy = fk.z * g10, ly = 0.f;
-                    for (int w = 0; w < n_pw; ++w) {
-                        const float2 pv = part[w * (nb << 5) + k];
-                        acc_two_sum(hx, lx, pv.x);
-                        acc_two_sum(hy, ly, pv.y);
-                    }
-                    float dx = (hx + lx) * s_f32[F_DTMU], dy = (hy + ly) * s_f32[F_DTMU];
-                    if (!isfinite(dx) || !isfinite(dy) || fmaxf(fabsf(dx), fabsf(dy)) > s_f32[F_DS]) bad = 1;
-                    float s, e, nh, nl;
-                    two_sum(xh[k], dx, s, e);
-                    two_sum(s, xl[k] + e, nh, nl);
-                    xh[k] = nh;
-                    xl[k] = nl;
-                    two_sum(yh[k], dy, s, e);
-                    two_sum(s, yl[k] + e, nh, nl);
-                    yh[k] = nh;
-                    yl[k] = nl;
+            for (int k = tid; k < n; k += T) {
+                // v_k = self term + the pair warps' partial sums, compensated
+                const float4 fk = ((const float4 *)src)[plane_b(k)];  // (Fx, ., Fy, .)
+                float hx = fk.x * g10, lx = 0.f, hy = fk.z * g10, ly = 0.f;
+                for (int w = 0; w < n_pw; ++w) {
+                    const float2 pv = part[w * (nb << 5) + k];
+                    acc_two_sum(hx, lx, pv.x);
+                    acc_two_sum(hy, ly, pv.y);
                 }
+                float dx = (hx + lx) * s_f32[F_DTMU], dy = (hy + ly) * s_f32[F_DTMU];
+                if (!isfinite(dx) || !isfinite(dy) || fmaxf(fabsf(dx), fabsf(dy)) > s_f32[F_DS]) bad = 1;
+                float s, e, nh, nl;
+                two_sum(xh[k], dx, s, e);
+                two_sum(s, xl[k] + e, nh, nl);
+                xh[k] = nh;
+                xl[k] = nl;
+                two_sum(yh[k], dy, s, e);
+                two_sum(s, yl[k] + e, nh, nl);
+                yh[k] = nh;
+                yl[k] = nl;
                 // the head point's observation: squared residual into J (FP64), trajectory row;
                 // obs_step is the same for every thread, so other steps branch around it
                 if (obs_step) {
                     if (!vel_obs(a, nh) && k == nf - 1) {
-                        double hxo = F64 ? sx[k] : (double)xh[k] + (double)xl[k];
-                        const double hyo = F64 ? sy[k] : (double)yh[k] + (double)yl[k];
+                        double hxo = (double)xh[k] + (double)xl[k];
+                        const double hyo = (double)yh[k] + (double)yl[k];
                         const long long o = obs_idx;
                         hxo += xref;
                         if (a.obs) {
@@ -1064,25 +848,20 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 if (TWO && a.obs_kind == SWIMMER_OBS_PAIR_DISTANCES) {
                     // distances between the tail tips and between the head centres (Sec. 4.2)
                     double c0x, c0y, c1x, c1y;
-                    head_centre<F64>(sx, sy, xh, xl, yh, yl, nf, nh, lane, c0x, c0y);
-                    head_centre<F64>(sx, sy, xh, xl, yh, yl, nsw + nf, nh, lane, c1x, c1y);
+                    head_centre(xh, xl, yh, yl, nf, nh, lane, c0x, c0y);
+                    head_centre(xh, xl, yh, yl, nsw + nf, nh, lane, c1x, c1y);
                     double tx, ty;
-                    if (F64) {
-                        tx = sx[nsw] - sx[0];
-                        ty = sy[nsw] - sy[0];
-                    } else {
-                        float hh, ll;
-                        df_sub(xh, xl, 0, nsw, hh, ll);
-                        tx = (double)hh + (double)ll;
-                        df_sub(yh, yl, 0, nsw, hh, ll);
-                        ty = (double)hh + (double)ll;
-                    }
+                    float hh, ll;
+                    df_sub(xh, xl, 0, nsw, hh, ll);
+                    tx = (double)hh + (double)ll;
+                    df_sub(yh, yl, 0, nsw, hh, ll);
+                    ty = (double)hh + (double)ll;
                     ox = sqrt(tx * tx + ty * ty);
                     oy = sqrt((c1x - c0x) * (c1x - c0x) + (c1y - c0y) * (c1y - c0y));
                 } else {
                     // head-centre velocity over the observation interval (Sec. 4.1)
                     double cx, cy;
-                    head_centre<F64>(sx, sy, xh, xl, yh, yl, nf, nh, lane, cx, cy);
+                    head_centre(xh, xl, yh, yl, nf, nh, lane, cx, cy);
                     const double inv = 1.0 / ((double)a.obs_every * a.dt);
                     ox = (cx - s_model[M_CX]) * inv;
                     oy = (cy - s_model[M_CY]) * inv;
@@ -1122,7 +901,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
             // (the first swimmer's, with two)
             const int k0 = nh > 0 ? nf : 0;
             double cx = 0.0;
-            for (int k = k0 + lane; k < nsw; k += 32) cx += F64 ? sx[k] : (double)xh[k] + (double)xl[k];
+            for (int k = k0 + lane; k < nsw; k += 32) cx += (double)xh[k] + (double)xl[k];
             for (int o = 16; o >= 1; o >>= 1) cx += __shfl_xor_sync(0xffffffffu, cx, o);
             if (tid == 0) {
                 const double c0 = nh > 0 ? L + (a.gap_over_ds + a.hr_over_ds) * ds - xref : 0.0;
@@ -1163,14 +942,11 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
 
 typedef void (*ForwardKernel)(FwdArgs);
 
-ForwardKernel forward_kernel_for(bool f64, const swimmer_config &c, bool big = false) {
+ForwardKernel forward_kernel_for(const swimmer_config &c, bool big = false) {
     const int model = c.n_swimmers == 2 ? 2 : c.n_head > 0 ? 1 : 0;
-    if (f64) return model == 2 ? forward_kernel<true, 2> : model == 1 ? forward_kernel<true, 1> : forward_kernel<true, 0>;
     if (big)
-        return model == 2 ? forward_kernel<false, 2, true>
-               : model == 1 ? forward_kernel<false, 1, true>
-                            : forward_kernel<false, 0, true>;
-    return model == 2 ? forward_kernel<false, 2> : model == 1 ? forward_kernel<false, 1> : forward_kernel<false, 0>;
+        return model == 2 ? forward_kernel<2, true> : model == 1 ? forward_kernel<1, true> : forward_kernel<0, true>;
+    return model == 2 ? forward_kernel<2> : model == 1 ? forward_kernel<1> : forward_kernel<0>;
 }
 
 }  // namespace
@@ -1288,18 +1064,18 @@ int upload_pair_units(swimmer_handle *h) {
 bool forward_fits(const swimmer_handle *h, int threads, int precision) {
     const bool f64 = precision == SWIMMER_FP64;
     const int P = handle_octaves(h) * (f64 ? F64_FINE : F32_SUB);
-    size_t smem = f64 ? smem_bytes<true>(h->cfg.n_max, P, threads) : smem_bytes<false>(h->cfg.n_max, P, threads);
+    const size_t smem = f64 ? forward64_smem(h->cfg.n_max, P, threads) : smem_bytes(h->cfg.n_max, P, threads);
     return smem + 1024 <= (size_t)h->max_smem;  // static shared memory of the kernel
 }
 
 // Samples the forward kernel holds at once on the device at its smallest launch shape (the
 // most resident samples); at least one per SM.
 int forward_slots(const swimmer_handle *h, int precision) {
-    const bool f64 = precision == SWIMMER_FP64;
     const int T = forward_min_threads(h, precision);
-    const int P = handle_octaves(h) * (f64 ? F64_FINE : F32_SUB);
-    size_t smem = f64 ? smem_bytes<true>(h->cfg.n_max, P, T) : smem_bytes<false>(h->cfg.n_max, P, T);
-    auto kern = forward_kernel_for(f64, h->cfg);
+    if (precision == SWIMMER_FP64) return std::max(1, forward64_resident(h, T)) * h->num_sms;
+    const int P = handle_octaves(h) * F32_SUB;
+    size_t smem = smem_bytes(h->cfg.n_max, P, T);
+    auto kern = forward_kernel_for(h->cfg);
     int per_sm = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
@@ -1391,8 +1167,17 @@ int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, do
     a.units = h->units;
     a.mode = f64 ? 0 : (shape & SHAPE_QUAD) ? 2 : (shape & SHAPE_WIDE) ? 1 : 0;
     a.tab_panels = handle_octaves(h) * (f64 ? F64_FINE : F32_SUB);
-    size_t smem = f64 ? smem_bytes<true>(a.n_max, a.tab_panels, T) : smem_bytes<false>(a.n_max, a.tab_panels, T);
-    auto kern = forward_kernel_for(f64, h->cfg);
+    if (f64) {
+        CUDA_TRY(cudaMemsetAsync(h->queue, 0, sizeof(int), s));
+        prof_k2_begin(h, s, B);
+        const int rc = launch_forward64(h, a, T, max_runs, s);
+        if (rc) return rc;
+        prof_k2_end(h, s);
+        prof_count(h, 1);
+        return 0;
+    }
+    size_t smem = smem_bytes(a.n_max, a.tab_panels, T);
+    auto kern = forward_kernel_for(h->cfg);
     CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   cudaSharedmemCarveoutMaxShared));
@@ -1407,10 +1192,10 @@ int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, do
     // FP32 with shared memory for so few threads per SM that each could hold 128 registers:
     // the instantiation compiled for that register budget (same CTAs per SM)
     // (with the table as 32-byte records, if that still fits)
-    const size_t smem_big = smem_bytes<false, true>(a.n_max, a.tab_panels, T);
-    if (!f64 && T <= 512 && per_sm >= 1 && (long long)per_sm * T * 128 <= h->regs_per_sm &&
+    const size_t smem_big = smem_bytes<true>(a.n_max, a.tab_panels, T);
+    if (T <= 512 && per_sm >= 1 && (long long)per_sm * T * 128 <= h->regs_per_sm &&
         smem_big + 1024 <= (size_t)h->max_smem) {
-        auto big = forward_kernel_for(f64, h->cfg, true);
+        auto big = forward_kernel_for(h->cfg, true);
         int per_big = 0;
         CUDA_TRY(cudaFuncSetAttribute(big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_big));
         CUDA_TRY(cudaFuncSetAttribute(big, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1422,7 +1207,7 @@ int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, do
         }
     }
     // four-target units need the 128-register budget; elsewhere the launch runs two-target ones
-    if (a.mode == 2 && kern == forward_kernel_for(f64, h->cfg)) a.mode = 1;
+    if (a.mode == 2 && kern == forward_kernel_for(h->cfg)) a.mode = 1;
     if (per_sm < 1) {
         set_error("forward kernel does not fit on an SM (threads %d, smem %zu)", T, smem);
         return SWIMMER_E_CUDA;

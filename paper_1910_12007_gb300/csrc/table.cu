@@ -694,7 +694,7 @@ table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scr
             double g1, g2;
             stokes_g(LITE ? p.delta * sqrt(node6_u(m) - 1.0) : p.delta * g_node[m].sig, p.delta, &g1, &g2);
             g1s[m] = g1;
-            g2s[m] = g2;
+            g2s[m] = LITE ? g2 : g2 * p.delta * p.delta;
         }
     } else if (LITE) {
         // A1 (prefix) and C (suffix) by warp 0: lanes own contiguous chunks (the order of these
@@ -751,7 +751,6 @@ table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scr
     } else {
         // A1 at node m: sum of the intervals up to it; C: the tail and the intervals beyond it.
         // Thread t owns the nodes [t chunk, (t + 1) chunk).
-        const double inv_d2 = 1.0 / (p.delta * p.delta);
         const int chunk = (M + K1_THREADS - 1) / K1_THREADS;
         const int lo = min(M, tid * chunk), hi = min(M, lo + chunk);
         double sa = 0.0, sc = 0.0;
@@ -783,8 +782,8 @@ table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scr
             const double a = g1s[m];
             g1s[m] = row[K1_E1 * (size_t)NODES_MAX + m] - row[K1_WA * (size_t)NODES_MAX + m] * a -
                      row[K1_WC * (size_t)NODES_MAX + m] * C;
-            g2s[m] = (row[K1_E2 * (size_t)NODES_MAX + m] - row[K1_VA * (size_t)NODES_MAX + m] * a -
-                      row[K1_VC * (size_t)NODES_MAX + m] * C) * inv_d2;
+            g2s[m] = row[K1_E2 * (size_t)NODES_MAX + m] - row[K1_VA * (size_t)NODES_MAX + m] * a -
+                     row[K1_VC * (size_t)NODES_MAX + m] * C;
         }
     }
     __syncthreads();
@@ -905,7 +904,9 @@ __global__ void kernel_eval_kernel(int m, const double *__restrict__ r, double *
             g1[i] = g2[i] = nan("");
             return;
         }
-        kern_f64(tab64, p.n_oct * F64_FINE - 1, u, g1[i], g2[i]);
+        double h;
+        kern_f64(tab64, p.n_oct * F64_FINE - 1, u, g1[i], h);
+        g2[i] = h / (p.delta * p.delta);
     } else {
         float inv_d2 = (float)(1.0 / (p.delta * p.delta));
         float r2 = (float)(rr * rr);

@@ -1,5 +1,5 @@
-// FP64 evaluation of a sample's kernel-function table (g1 = B'', g2 = (r B'' - B')/r^3,
-// Eq. BrV) with almost no FP64 instruction.  GB300 issues an FP64 instruction of a warp every 16
+// FP64 evaluation of a sample's kernel-function table (g1 = B'' and h = delta^2 g2,
+// g2 = (r B'' - B')/r^3, Eq. BrV) with almost no FP64 instruction.  GB300 issues an FP64 instruction of a warp every 16
 // clocks of an SM and an FP32 one every quarter clock, so a degree-9 Clenshaw recurrence for two
 // functions (36 FP64 FMAs) is what a pair evaluation used to wait for.
 //
@@ -12,8 +12,8 @@
 // functions run in the two halves of the packed FP32 instructions.  1024 FP64 runs of N = 128, 200
 // steps: 321 -> 109 ms; a lone run of N = 64, 2000 steps: 133 -> 53 ms.
 //
-// Record of a panel (F64_REC float4): {c0 of g1, c0 of g2} as doubles; for k = 1 .. 5 the high
-// parts of c_k of g1 and g2, then the low parts; c6 of g1, g2, c7 of g1, g2.
+// Record of a panel (F64_REC float4): {c0 of g1, c0 of h} as doubles; for k = 1 .. 5 the high
+// parts of c_k of g1 and h, then the low parts; c6 of g1, h, c7 of g1, h.
 #pragma once
 
 #include "common.cuh"
@@ -91,12 +91,12 @@ static __device__ __forceinline__ double poly1_f64(const float4 *__restrict__ re
 }
 
 static __device__ __forceinline__ void kern_f64(const float4 *__restrict__ tab, int pmax, double u, double &g1,
-                                                double &g2) {
+                                                double &h) {
     float th, tl;
     const float4 *rec = tab + F64_REC * panel_f64(u, pmax, th, tl);
     const double2 c0 = *(const double2 *)rec;
     float2 qh, ql;
     poly_f64(rec, th, tl, qh, ql);
     g1 = c0.x + (widen(qh.x) + widen(ql.x));
-    g2 = c0.y + (widen(qh.y) + widen(ql.y));
+    h = c0.y + (widen(qh.y) + widen(ql.y));
 }
