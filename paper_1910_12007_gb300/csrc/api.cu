@@ -196,8 +196,6 @@ extern "C" int swimmer_init(const swimmer_config *cfg, swimmer_handle **out) {
     ALLOC(h->run_work, B);
     ALLOC(h->surr_norm, 2 * SWIMMER_MLP_OUT);
     ALLOC(h->surr_params, SWIMMER_MLP_NPARAM);
-    ALLOC(h->surr_x, (size_t)B * SWIMMER_MLP_IN);
-    ALLOC(h->surr_y, (size_t)B * SWIMMER_MLP_OUT);
     {
         cudaError_t e1 = cudaMallocHost((void **)&h->host_pinned, (B + 128) * sizeof(int));
         cudaError_t e2 = cudaMallocHost((void **)&h->host_pinned_d, 64 * sizeof(double));
@@ -233,7 +231,7 @@ extern "C" int swimmer_destroy(swimmer_handle *h) {
                     h->tmpl_master, h->tmpl_map, h->p_accept_dev, h->stage_q, h->stage_summary, h->surr_dstat,
                     h->surr_trust, h->cum, h->info,
                     h->work, h->run_work,
-                    h->surr_norm, h->surr_params, h->surr_x, h->surr_y, h->surr_ws, h->units};
+                    h->surr_norm, h->surr_params, h->surr_frag, h->units};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (h->host_pinned) cudaFreeHost(h->host_pinned);

@@ -143,8 +143,7 @@ struct swimmer_handle {
     int surr_obs_stride;
     double surr_log10_kt, surr_omega;
     int surr_ready;
-    float *surr_x, *surr_y; // [b_max][5], [b_max][80]
-    float *surr_ws;         // MLP workspace for b_max samples (allocated by swimmer_surrogate_set)
+    uint4 *surr_frag;       // the same as MMA fragments (allocated by swimmer_surrogate_set)
 };
 
 // ---- error reporting -----------------------------------------------------------------
