@@ -615,7 +615,7 @@ table_nodes_kernel(const SampleParams *__restrict__ sp, double *__restrict__ scr
     // ---- the node: g1 = E1 - WA A1 - WC C, delta^2 g2 = E2 - VA A1 - VC C
     const double x = beta * nd.sig, rs = rsb * nd.rsq, z = rs * rs;
     double i0, i2, k0, k2, t2k2, ix2w;  // t2k2 = 2/x^2 - K2, ix2w = 1/x^2 - (K0 + K2)/2
-    const double y = 0.25 * x * x, lx = lb + nd.lns;
+    const double y = 0.25 * x * x;
     if (x <= I_SERIES) {
         if (x <= 2.0) {
             i0 = horner<SER_K>(c_i0, y);
@@ -630,6 +630,7 @@ table_nodes_kernel(const SampleParams *__restrict__ sp, double *__restrict__ scr
         i2 = ex * i_poly(c_i2p, c_i2q, x > I_SPLIT, z);
     }
     if (x <= 2.0) {
+        const double lx = log(0.5 * x) + EGAMMA;  // (the sum lb + ln sigma would round twice more)
         k0 = fma(-lx, i0, y * horner<SER_K - 1>(c_k0t + 1, y));
         // 2/x^2 - K2 = 1/2 + y sum_k [lx - (H_k + H_{k+2})/2] y^k/(k! (k+2)!)
         t2k2 = fma(y, fma(lx, i2, -horner<SER_K>(c_t2, y)), 0.5);
@@ -795,19 +796,22 @@ table_build_kernel(SampleParams *__restrict__ sp, const double *__restrict__ scr
             const int panel = q % np, part = q / np;
             float4 *rec = t64 + F64_REC * (panel * F64_SPLIT + part);
             const double *ga = g1s + panel * F64_NODES, *gb = g2s + panel * F64_NODES;
+            // the fit of the differences from a middle node: they are exact, and the rounding of
+            // the higher coefficients' sums of alternating terms stays in proportion to them
+            const double ma = ga[F64_NODES / 2], mb = gb[F64_NODES / 2];
             double ca[F64_COEF], cb[F64_COEF];
 #pragma unroll
             for (int k = 0; k < F64_COEF; ++k) {
                 double x = 0.0, y = 0.0;
                 for (int i = 0; i < F64_NODES; ++i) {
                     const double w = c_fit64[part][k][i];
-                    x = fma(w, ga[i], x);
-                    y = fma(w, gb[i], y);
+                    x = fma(w, ga[i] - ma, x);
+                    y = fma(w, gb[i] - mb, y);
                 }
                 ca[k] = x;
                 cb[k] = y;
             }
-            *(double2 *)rec = make_double2(ca[0], cb[0]);
+            *(double2 *)rec = make_double2(ma + ca[0], mb + cb[0]);
 #pragma unroll
             for (int k = 1; k <= 5; ++k) {
                 const float ha = (float)ca[k], hb = (float)cb[k];
