@@ -1111,17 +1111,57 @@ int forward_threads(const swimmer_handle *h, int B, int precision) {
     const int tT = tuned & SHAPE_THREADS;
     int T = forward_min_threads(h, precision);
     if (tT >= T && tT <= 1024 && forward_fits(h, tT, precision)) return tuned;
-    int cap = 1024;
-    if (precision != SWIMMER_FP64) {  // warps beyond the pair units only help the O(N) phases
-        const int nbm = (h->cfg.n_max + 31) / 32;
-        while (cap > T && cap / 2 >= 32 * nbm * nbm) cap /= 2;
+    const int n = h->cfg.n_max, nbm = (n + 31) / 32;
+    if (precision == SWIMMER_FP64) {
+        // the pair sum gives a target floor(T / n) threads: the smallest count of two a target or more
+        // that leaves at most a seventh of the threads without one (else the best), and eight warps
+        // for a run alone on its SM.  1024 runs, us a step: N = 100 512 threads 324, 128 (22 % idle)
+        // 389; N = 148 512 663, 256 (42 % idle) 706; N = 128 256 486, 128 492 to 552; N = 64, 100 runs:
+        // 256 20.9, 128 23.0, 1024 22.8.
+        int best = 0, best_t = T, t = bucket == 0 ? 256 : 128;
+        while (t < 2 * n && t < 1024) t <<= 1;
+        for (; t <= 1024 && forward_fits(h, t, precision); t <<= 1) {
+            const int used = 1024 / t * (t / n * n);  // of 1024 threads
+            if (used > best) {
+                best = used;
+                best_t = t;
+            }
+            if (7 * (1024 - used) <= 1024) break;
+        }
+        return best_t;
     }
+    // FP32, the flagellum of 4 blocks of 32 points and more (us a step of 100, 300, 600 and 1100 runs
+    // by shape: threads, w two-target, q four-target units).  Below 8 blocks a run alone on its SM or
+    // one of two takes 256 threads, more share the SM at 128: N = 128 256w 3.2, 4.5, 8.2, 16.0, 128w
+    // 4.0, 4.8, 7.5, 16.0, and from six runs per SM on four at a time at 128 registers (128q, whose
+    // lists are the two-target ones here) beat five to seven at 64: 1100 runs of N = 128 14.6, of
+    // N = 192 29.3 against 32.3, of N = 224 38.2 against 42.4.  From 8 blocks on four-target units and 16 warps of 128 registers an
+    // SM, as one run, as two, or (8 and 9 blocks) as four: N = 256 512q 7.3, 14.5, 28.8, 57.3, 256q 7.7,
+    // 12.4, 24.5, 48.5, 128q ., 13.3, 23.1, 46.0; N = 512 512q 24.4, 48.5, 96.5, 192, 256q 25.7, 44.8,
+    // 87.4, 170; from about 700 points two runs' shared memory no longer fits: N = 768 512q 49.7,
+    // 99.3, 198, 256q 53.2, 106, 212.  (The rule before took two-target units and as many threads as
+    // the batch leaves: N = 512 31.4, 52.7, 92.5, 236.)
+    if (h->cfg.n_head == 0 && nbm >= 4) {
+        int shape;
+        if (nbm < 8) {
+            shape = bucket <= 1 ? 256 | SHAPE_WIDE : bucket <= 4 ? 128 | SHAPE_WIDE : 128 | SHAPE_QUAD;
+        } else if (bucket == 0) {
+            shape = 512 | SHAPE_QUAD;
+        } else if (nbm <= 9 && bucket >= 2) {
+            shape = 128 | SHAPE_QUAD;
+        } else {
+            const size_t smem = smem_bytes<true>(n, handle_octaves(h) * F32_SUB, 256);
+            shape = (2 * (smem + 1536) <= (size_t)h->max_smem + 1024 ? 256 : 512) | SHAPE_QUAD;
+        }
+        if (forward_fits(h, shape & SHAPE_THREADS, precision)) return shape;
+    }
+    int cap = 1024;  // warps beyond the pair units only help the O(N) phases
+    while (cap > T && cap / 2 >= 32 * nbm * nbm) cap /= 2;
     while (T < cap && (long long)B * T * 2 <= (long long)h->num_sms * 1024 && forward_fits(h, 2 * T, precision))
         T <<= 1;
-    // two-target units (measured): from 8 blocks of 32 points at every thread count, and from 4
-    // blocks when the batch fills the GPU (the heuristic stays at 128 threads only then)
-    const int nbm = (h->cfg.n_max + 31) / 32;
-    if (precision != SWIMMER_FP64 && (nbm >= 8 || (nbm >= 4 && T == 128))) return T | SHAPE_WIDE;
+    // two-target units from 8 blocks of 32 points at every thread count, and from 4 blocks when the
+    // batch fills the GPU (the heuristic stays at 128 threads only then)
+    if (nbm >= 8 || (nbm >= 4 && T == 128)) return T | SHAPE_WIDE;
     return T;
 }
 
@@ -1195,7 +1235,11 @@ int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, do
     // FP32 with shared memory for so few threads per SM that each could hold 128 registers:
     // the instantiation compiled for that register budget (same CTAs per SM)
     // (with the table as 32-byte records, if that still fits)
+    // (four-target units are for that instantiation only: their launches hold fewer CTAs per SM
+    // when that many registers need it)
     const size_t smem_big = smem_bytes<true>(a.n_max, a.tab_panels, T);
+    if (a.mode == 2 && T <= 512 && smem_big + 1024 <= (size_t)h->max_smem)
+        per_sm = min(per_sm, max(1, h->regs_per_sm / (128 * T)));
     if (T <= 512 && per_sm >= 1 && (long long)per_sm * T * 128 <= h->regs_per_sm &&
         smem_big + 1024 <= (size_t)h->max_smem) {
         auto big = forward_kernel_for(h->cfg, true);
