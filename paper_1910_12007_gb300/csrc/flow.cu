@@ -6,11 +6,10 @@
 //
 // Bound by the FP64 pipe (16 clocks a warp instruction).  One thread per target; the sample's
 // table, the pressure kernel's (delta^2 G_delta'/r is a function of u = 1 + r^2/delta^2 alone, made
-// once per device in the same form) and the sources sit in shared memory, so a pair takes 19 FP64
-// instructions: separation and u 5, the three kernel functions 2 each, the sums 8.  With the
+// once per device in the same form) and the sources sit in shared memory, so a pair takes 16 FP64
+// instructions: separation and u 5, the three kernel functions one each, the sums 8.  With the
 // Clenshaw recurrences, square root and division in FP64 and the table read from L1 it took 75
-// (512 x 512 targets and 74 points: 2.8 ms a call, of it 2.75 here; now 0.75 ms a call, 0.66
-// here).  CTAs are persistent: one or two per SM load the tables once and walk the targets.
+// (512 x 512 targets and 74 points: 2.8 ms a call, of it 2.75 here; now 0.65 ms a call).  CTAs are persistent: one or two per SM load the tables once and walk the targets.
 #include <math.h>
 #include <string.h>
 
@@ -80,7 +79,7 @@ __global__ void __launch_bounds__(FLOW_THREADS) flow_kernel(int n, const double 
                     const double2 c0 = *(const double2 *)rec;
                     float2 qh, ql;
                     poly_f64(rec, th, tl, qh, ql);
-                    const double g1 = c0.x + (widen(qh.x) + widen(ql.x)), w = fd * (c0.y + (widen(qh.y) + widen(ql.y)));
+                    const double g1 = c0.x + join(qh.x, ql.x), w = fd * (c0.y + join(qh.y, ql.y));
                     ax = fma(F.x, g1, ax);
                     ay = fma(F.y, g1, ay);
                     vx = fma(w, dx, vx);

@@ -4,8 +4,8 @@
 // Bound by the FP64 pipe: GB300 issues a warp's FP64 instruction every 16 clocks of an SM, 64 times
 // slower than FP32.  So
 //   - positions are kept in units of delta (u = 1 + |e|^2 takes two FMAs), and the kernel functions
-//     come from table_eval.cuh with two FP64 additions each: 15 FP64 instructions per ordered pair
-//     (separation 2, u 2, kernel functions 4, F . e and its product 3, the sums 4) where two
+//     come from table_eval.cuh with one FP64 addition each: 13 FP64 instructions per ordered pair
+//     (separation 2, u 2, kernel functions 2, F . e and its product 3, the sums 4) where two
 //     Clenshaw recurrences took 54;
 //   - the threads that share a target leave their partial sums in shared memory and one thread adds
 //     them and updates the point: as warp shuffles, additions and the update cost their 16 clocks in
