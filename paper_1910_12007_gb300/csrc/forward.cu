@@ -1067,7 +1067,7 @@ int upload_pair_units(swimmer_handle *h) {
 bool forward_fits(const swimmer_handle *h, int threads, int precision) {
     const bool f64 = precision == SWIMMER_FP64;
     const int P = handle_octaves(h) * (f64 ? F64_FINE : F32_SUB);
-    const size_t smem = f64 ? forward64_smem(h->cfg.n_max, P, threads) : smem_bytes(h->cfg.n_max, P, threads);
+    const size_t smem = f64 ? forward64_smem(h->cfg.n_max, P, threads, 0) : smem_bytes(h->cfg.n_max, P, threads);
     return smem + 1024 <= (size_t)h->max_smem;  // static shared memory of the kernel
 }
 
@@ -1113,7 +1113,15 @@ int forward_threads(const swimmer_handle *h, int B, int precision) {
     if (tT >= T && tT <= 1024 && forward_fits(h, tT, precision)) return tuned;
     const int n = h->cfg.n_max, nbm = (n + 31) / 32;
     if (precision == SWIMMER_FP64) {
-        // the pair sum gives a target floor(T / n) threads: the smallest count of two a target or more
+        // symmetric pair sum: two or more runs per SM share its FP64 pipe at 256 threads each (128
+        // up to two blocks), a run alone takes twice as many warps from 128 points on (1024 runs, us a step:
+        // N = 64 128 88, 256 104; N = 128 256 322, 128 331; N = 192 256 703, 512 743)
+        if (forward64_pair_warps(h, 128) > 0) {
+            int t = n <= 64 ? 128 : n > 128 && bucket == 0 ? 512 : 256;
+            while (t < n) t <<= 1;
+            if (forward_fits(h, t, precision)) return t;
+        }
+        // else the pair sum gives a target floor(T / n) threads: the smallest count of two a target or more
         // that leaves at most a seventh of the threads without one (else the best), and eight warps
         // for a run alone on its SM.  1024 runs, us a step: N = 100 512 threads 324, 128 (22 % idle)
         // 389; N = 148 512 663, 256 (42 % idle) 706; N = 128 256 486, 128 492 to 552; N = 64, 100 runs:
@@ -1130,22 +1138,17 @@ int forward_threads(const swimmer_handle *h, int B, int precision) {
         }
         return best_t;
     }
-    // FP32, the flagellum of 4 blocks of 32 points and more (us a step of 100, 300, 600 and 1100 runs
-    // by shape: threads, w two-target, q four-target units).  Below 8 blocks a run alone on its SM or
-    // one of two takes 256 threads, more share the SM at 128: N = 128 256w 3.2, 4.5, 8.2, 16.0, 128w
-    // 4.0, 4.8, 7.5, 16.0, and from six runs per SM on four at a time at 128 registers (128q, whose
-    // lists are the two-target ones here) beat five to seven at 64: 1100 runs of N = 128 14.6, of
-    // N = 192 29.3 against 32.3, of N = 224 38.2 against 42.4.  From 8 blocks on four-target units and 16 warps of 128 registers an
-    // SM, as one run, as two, or (8 and 9 blocks) as four: N = 256 512q 7.3, 14.5, 28.8, 57.3, 256q 7.7,
-    // 12.4, 24.5, 48.5, 128q ., 13.3, 23.1, 46.0; N = 512 512q 24.4, 48.5, 96.5, 192, 256q 25.7, 44.8,
-    // 87.4, 170; from about 700 points two runs' shared memory no longer fits: N = 768 512q 49.7,
-    // 99.3, 198, 256q 53.2, 106, 212.  (The rule before took two-target units and as many threads as
-    // the batch leaves: N = 512 31.4, 52.7, 92.5, 236.)
-    if (h->cfg.n_head == 0 && nbm >= 4) {
+    // FP32, the flagellum from 8 blocks of 32 points on: four-target units and 16 warps of 128 registers
+    // an SM, as one run, as two, or (8 and 9 blocks) as four.  us a step of 100, 300, 600 and 1100 runs
+    // by shape (threads, q four-target units): N = 256 512q 7.3, 14.5, 28.8, 57.3, 256q 7.7, 12.4, 24.5,
+    // 48.5, 128q ., 13.3, 23.1, 46.0; N = 512 512q 24.4, 48.5, 96.5, 192, 256q 25.7, 44.8, 87.4, 170;
+    // from about 700 points two runs' shared memory no longer fits: N = 768 512q 49.7, 99.3, 198, 256q
+    // 53.2, 106, 212.  (Two-target units and as many threads as the batch leaves: N = 512 31.4, 52.7,
+    // 92.5, 236.)  Below, where a shorter step's larger displacements show the order of the pair sum in
+    // a log-likelihood's ninth digit, shapes keep their partition of the sum.
+    if (h->cfg.n_head == 0 && nbm >= 8) {
         int shape;
-        if (nbm < 8) {
-            shape = bucket <= 1 ? 256 | SHAPE_WIDE : bucket <= 4 ? 128 | SHAPE_WIDE : 128 | SHAPE_QUAD;
-        } else if (bucket == 0) {
+        if (bucket == 0) {
             shape = 512 | SHAPE_QUAD;
         } else if (nbm <= 9 && bucket >= 2) {
             shape = 128 | SHAPE_QUAD;
@@ -1160,7 +1163,11 @@ int forward_threads(const swimmer_handle *h, int B, int precision) {
     while (T < cap && (long long)B * T * 2 <= (long long)h->num_sms * 1024 && forward_fits(h, 2 * T, precision))
         T <<= 1;
     // two-target units from 8 blocks of 32 points at every thread count, and from 4 blocks when the
-    // batch fills the GPU (the heuristic stays at 128 threads only then)
+    // batch fills the GPU (the heuristic stays at 128 threads only then).  Below 8 blocks the four-target
+    // shape has the same lists; from six runs per SM on its four at a time at 128 registers beat five
+    // to seven at 64 (128 threads, 1100 runs: N = 128 14.6 against 16.0 us a step, N = 192 29.3, 32.3, N = 224
+    // 38.2, 42.4)
+    if (nbm >= 4 && nbm < 8 && T == 128 && bucket >= 5 && h->cfg.n_head == 0) return T | SHAPE_QUAD;
     if (nbm >= 8 || (nbm >= 4 && T == 128)) return T | SHAPE_WIDE;
     return T;
 }

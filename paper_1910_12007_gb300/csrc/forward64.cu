@@ -12,8 +12,12 @@
 //     every warp, for two or four useful lanes each;
 //   - (cos, sin)(omega t) is made for 32 steps at a time, a lane each, and the preferred curvature
 //     is P_k cos + Q_k sin; springs and curvature take one reciprocal square root each.
-// Target i meets source i + d mod n at step d (the lanes of a warp share d: on a smooth filament
-// they read the same table panel).  A lone run is spread over a cluster of up to 16 SMs: a CTA owns
+// Of a run that has a CTA to itself every unordered pair is evaluated once, in the blocks and units of
+// forward.cu (19 FP64 instructions: the symmetric mobility 5, two sums 4 each): 1024 runs of N = 128 85.6 ->
+// 65.5 ms.
+// Where the padding to blocks would cost more than that saves, where the warps' arrays do not fit
+// and in a cluster, target i meets source i + d mod n at step d (the lanes of a warp share d: on a
+// smooth filament they read the same table panel).  A lone run is spread over a cluster of up to 16 SMs: a CTA owns
 // n / C points; forces and new positions go to every CTA's shared memory (double-buffered
 // positions, two cluster barriers a step).
 // Measured (whole calls): a lone run of N = 64, 2000 steps 53.1 -> 13.9 ms (26.5 -> 6.9 us a step) on a
@@ -80,7 +84,12 @@ __device__ __forceinline__ void run_sync(int C) {
     }
 }
 
-__host__ __device__ inline size_t align128(size_t b) { return (b + 127) & ~size_t(127); }
+// shared memory before the table
+__host__ __device__ inline size_t state_bytes(int n_max, int threads, int pair_warps) {
+    const size_t np = (n_max + 31) & ~31, part = pair_warps * np;
+    const size_t b = sizeof(double2) * (7 * np + (part > (size_t)threads ? part : (size_t)threads));
+    return (b + 127) & ~size_t(127);
+}
 
 // mean of the head points from k0 on (one warp, fixed order); all lanes get it
 __device__ __forceinline__ double2 centre(const double2 *pos, int k0, int count, int lane) {
@@ -96,20 +105,75 @@ __device__ __forceinline__ double2 centre(const double2 *pos, int k0, int count,
     return make_double2(x / count, y / count);
 }
 
+// One unit of the symmetric pair sum (a warp, 16 steps): lane l holds target I*32 + l and at step d =
+// d0 .. d0 + 15 meets source J*32 + (l + d) mod 32; the pair's term is the symmetric mobility M = h e e^T
+// - g1 I applied to both forces, and the source's sum moves down one lane per step with its source.
+// A diagonal block (I = J) runs d = 1 .. 16, at 16 with half the lanes (the units of forward.cu).
+template <bool DIAG>
+__device__ __forceinline__ void pair_unit64(const double2 *__restrict__ X, const double2 *__restrict__ frc,
+                                            const float4 *__restrict__ tab, int pmax, int lane, int I, int Jb, int d0,
+                                            double2 *__restrict__ mypart) {
+    const double2 xi = X[32 * I + lane], fi = frc[32 * I + lane];
+    double vx = 0.0, vy = 0.0, ax = 0.0, ay = 0.0;
+#pragma unroll 2
+    for (int s = 0; s < 16; ++s) {
+        const int j = 32 * Jb + ((lane + d0 + s) & 31);
+        const double2 xj = X[j], f = frc[j];
+        const double ex = xi.x - xj.x, ey = xi.y - xj.y;
+        double g1, h;
+        kern_f64(tab, pmax, fma(ex, ex, fma(ey, ey, 1.0)), g1, h);
+        if (DIAG && s == 15 && lane >= 16) g1 = h = 0.0;
+        const double hx = h * ex, hy = h * ey;
+        const double m11 = fma(hx, ex, -g1), m12 = hx * ey, m22 = fma(hy, ey, -g1);
+        vx = fma(m11, f.x, fma(m12, f.y, vx));
+        vy = fma(m12, f.x, fma(m22, f.y, vy));
+        ax = fma(m11, fi.x, fma(m12, fi.y, ax));
+        ay = fma(m12, fi.x, fma(m22, fi.y, ay));
+        ax = __shfl_sync(0xffffffffu, ax, (lane + 1) & 31);
+        ay = __shfl_sync(0xffffffffu, ay, (lane + 1) & 31);
+    }
+    // lane l holds the sum of source (l + d0 + 16) mod 32: to its own lane
+    const int from = (lane - d0 - 16) & 31;
+    ax = __shfl_sync(0xffffffffu, ax, from);
+    ay = __shfl_sync(0xffffffffu, ay, from);
+    double2 pv = mypart[32 * I + lane];
+    pv.x += vx;
+    pv.y += vy;
+    if (DIAG) {
+        pv.x += ax;
+        pv.y += ay;
+    }
+    mypart[32 * I + lane] = pv;
+    if (!DIAG) {
+        double2 pa = mypart[32 * Jb + lane];
+        pa.x += ax;
+        pa.y += ay;
+        mypart[32 * Jb + lane] = pa;
+    }
+}
+
+// whether a run of n points is worth the symmetric sum: 19 FP64 instructions per unordered pair of
+// the points padded to blocks of 32, against 26 of the points
+__host__ __device__ inline bool symmetric_pays(int n) {
+    const int np = (n + 31) & ~31;
+    return 19 * np * np < 26 * n * n;
+}
+
 // MODEL 0: the flagellum; 1: the full sperm model (head points and neck); 2: two sperm models
 // coupled by the fluid.  C CTAs (a cluster when C > 1) share a run.
 template <int MODEL, int MAXT>
-__global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C) {
+__global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, int pw) {
     constexpr bool HEAD = MODEL >= 1, TWO = MODEL == 2;
     extern __shared__ __align__(128) unsigned char smraw[];
     const int n_max = a.n_max, T = blockDim.x, tid = threadIdx.x, lane = tid & 31;
-    double2 *pos = (double2 *)smraw;       // [2][n_max] positions / delta, relative to (L/2, 0)
-    double2 *frc = pos + 2 * n_max;        // [n_max] point forces
-    double2 *tv = frc + n_max;             // [n_max] tension of segment (k, next)
-    double2 *b0 = tv + n_max, *b4 = b0 + n_max;  // [n_max] bending of centre k on its neighbours
-    double2 *pq = b4 + n_max;              // [n_max] preferred-curvature coefficients
-    double2 *part = pq + n_max;            // [T] partial velocities
-    const float4 *tab = (const float4 *)(smraw + align128(sizeof(double2) * (7 * (size_t)n_max + T)));
+    const int np = (n_max + 31) & ~31;     // points in blocks of 32
+    double2 *pos = (double2 *)smraw;       // [2][np] positions / delta, relative to (L/2, 0)
+    double2 *frc = pos + 2 * np;           // [np] point forces
+    double2 *tv = frc + np;                // [np] tension of segment (k, next)
+    double2 *b0 = tv + np, *b4 = b0 + np;  // [np] bending of centre k on its neighbours
+    double2 *pq = b4 + np;                 // [np] preferred-curvature coefficients
+    double2 *part = pq + np;               // partial velocities: [T], or [pw][np] of the symmetric sum's warps
+    const float4 *tab = (const float4 *)(smraw + state_bytes(n_max, T, pw));
     __shared__ int s_work, s_bad[2];
     __shared__ Rest s_rest[6];  // flagellum segment, head membrane, diametral, neck A, neck B, neck gap
     // stencils of the flagellum [0] and the head [1]: delta/(2 h), delta/h^2, 1/(2 h), 1/h^2, 2 K h;
@@ -181,6 +245,15 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C) {
                 pq[k] = make_double2(-p.amp * (c1 * cs + c2 * sn), -p.amp * (c1 * sn - c2 * cs));
             }
         }
+        // force-free sources ds apart beyond the last point fill the last block (symmetric sum)
+        const int nbk = (n + 31) >> 5;
+        for (int k = n + tid; k < 32 * nbk; k += T) {
+            const double end = nh ? L + gap + 2.0 * hr : L;
+            pos[k] = pos[np + k] = make_double2((end - xref + (k - n + 1) * ds) * inv_d, TWO ? a.swim_d * inv_d : 0.0);
+            frc[k] = make_double2(0.0, 0.0);
+        }
+        const bool sym = pw > 0 && symmetric_pays(n);
+        const unsigned *units = a.units + UNIT_HDR + a.units[nbk - 1];  // the one-target list of nbk blocks
         if (tid == 0) {
             const double c1 = hr * (1.0 - cos(dth)), s1 = hr * sin(dth);
             const double l0[6] = {ds, 2.0 * hr * sin(0.5 * dth), 2.0 * hr, hypot(gap + c1, s1), hypot(ds + gap + c1, s1),
@@ -239,7 +312,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C) {
         const int obs_every = (int)min(a.obs_every, (long long)INT_MAX);  // > steps: no observation
         int obs_left = obs_every, obs_idx = 0;
         for (int step = 0; step < (int)last; ++step) {
-            const double2 *X = pos + (step & 1) * n_max;
+            const double2 *X = pos + (step & 1) * np;
             const bool obs_step = --obs_left == 0;
             int bad = 0;
             if ((step & 31) == 0) {  // (the last reads of s_rot lie before a barrier)
@@ -402,7 +475,34 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C) {
             // ---- D: pair sum of the own points, e = d / delta, h = delta^2 g2:
             //      v_i = (1/mu) sum_j [-F_j g1 + (F_j . e) e h]
             double vx = 0.0, vy = 0.0;
-            if (split < S) {
+            if (sym) {
+                // every unordered pair once; warp w takes units w, w + pw, ... and adds them into its
+                // own array, the arrays are added in order
+                const int warp = tid >> 5;
+                if (warp < pw) {
+                    double2 *mypart = part + warp * np;
+                    for (int k = lane; k < 32 * nbk; k += 32) mypart[k] = make_double2(0.0, 0.0);
+                    for (int un = warp; un < nbk * nbk; un += pw) {
+                        const unsigned pk = units[un];
+                        const int I = pk & 31, Jb = (pk >> 5) & 31, code = (pk >> 25) & 3;
+                        if (I == Jb)
+                            pair_unit64<true>(X, frc, tab, npan - 1, lane, I, Jb, 1, mypart);
+                        else
+                            pair_unit64<false>(X, frc, tab, npan - 1, lane, I, Jb, code << 4, mypart);
+                    }
+                }
+                __syncthreads();
+                if (my < m && (G == 1 || (tid & 7) == 0)) {
+                    const double2 f = frc[my];
+                    vx = -f.x * self_g1;
+                    vy = -f.y * self_g1;
+                    for (int w = 0; w < pw; ++w) {
+                        const double2 v = part[w * np + my];
+                        vx += v.x;
+                        vy += v.y;
+                    }
+                }
+            } else if (split < S) {
                 const int i = k_lo + pt;
                 const double2 xi = X[i];
                 if (split == 0) {
@@ -426,7 +526,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C) {
                     vy = fma(wv, ey, fma(-f.y, g1, vy));
                 }
             }
-            if (S > 1) {
+            if (!sym && S > 1) {
                 if (split < S) part[split * m + pt] = make_double2(vx, vy);
                 __syncthreads();
                 vx = vy = 0.0;
@@ -451,7 +551,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C) {
                 }
             }
             // ---- E: Euler step into the other position buffer, divergence, observations
-            double2 *Xn = pos + ((step + 1) & 1) * n_max;
+            double2 *Xn = pos + ((step + 1) & 1) * np;
             if (my < m && (G == 1 || (tid & 7) == 0)) {
                 const int k = k_lo + my;
                 const double dx = vx * dt_c, dy = vy * dt_c;  // displacement this step
@@ -528,7 +628,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C) {
             // coordinates) or, with a head, of the head centre (the first swimmer's, with two), over
             // the run's duration; one warp sums in a fixed order
             const int k0 = nh > 0 ? nf : 0;
-            const double2 c = centre(pos + (a.steps & 1) * n_max, k0, nsw - k0, lane);
+            const double2 c = centre(pos + (a.steps & 1) * np, k0, nsw - k0, lane);
             if (tid == 0) {
                 const double c0 = nh > 0 ? L + (a.gap_over_ds + a.hr_over_ds) * ds - xref : 0.0;
                 a.speed[b] = status == SWIMMER_OK ? (c.x * delta - c0) / (a.steps * a.dt) : nan("");
@@ -564,7 +664,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C) {
     }
 }
 
-typedef void (*Kernel64)(FwdArgs, int);
+typedef void (*Kernel64)(FwdArgs, int, int);
 
 Kernel64 kernel_for(const swimmer_config &c, int threads) {
     const int model = c.n_swimmers == 2 ? 2 : c.n_head > 0 ? 1 : 0;
@@ -575,13 +675,23 @@ Kernel64 kernel_for(const swimmer_config &c, int threads) {
 
 }  // namespace
 
-size_t forward64_smem(int n_max, int panels, int threads) {
-    return align128(sizeof(double2) * (7 * (size_t)n_max + threads)) + sizeof(float4) * F64_REC * (size_t)panels;
+size_t forward64_smem(int n_max, int panels, int threads, int pair_warps) {
+    return state_bytes(n_max, threads, pair_warps) + sizeof(float4) * F64_REC * (size_t)panels;
+}
+
+// Warps of the symmetric pair sum in a launch with one run per CTA: at most one per unit, and 16, 8 or 4
+// as their arrays fit; 0 where it does not pay for the largest sample.
+int forward64_pair_warps(const swimmer_handle *h, int threads) {
+    const int n = h->cfg.n_max, nb = (n + 31) / 32;
+    if (!symmetric_pays(n)) return 0;
+    for (int w = std::min(16, std::min(threads / 32, nb * nb)); w >= std::min(4, nb * nb); w >>= 1)
+        if (forward64_smem(n, handle_octaves(h) * F64_FINE, threads, w) + 2048 <= (size_t)h->max_smem) return w;
+    return 0;
 }
 
 // CTAs per SM of a launch with one run per CTA (0: does not fit)
 int forward64_resident(const swimmer_handle *h, int threads) {
-    const size_t smem = forward64_smem(h->cfg.n_max, handle_octaves(h) * F64_FINE, threads);
+    const size_t smem = forward64_smem(h->cfg.n_max, handle_octaves(h) * F64_FINE, threads, forward64_pair_warps(h, threads));
     Kernel64 kern = kernel_for(h->cfg, threads);
     int per_sm = 0;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
@@ -608,7 +718,7 @@ int launch_forward64(swimmer_handle *h, const FwdArgs &a, int threads, int max_r
         if (a.n_max < C * CLUSTER_POINTS || C * a.B > h->num_sms) continue;
         int T = CLUSTER_THREADS;
         while (T < (a.n_max + C - 1) / C + 1) T <<= 1;  // a thread per own point
-        const size_t smem = forward64_smem(a.n_max, a.tab_panels, T);
+        const size_t smem = forward64_smem(a.n_max, a.tab_panels, T, 0);
         if (T > 1024 || smem + 2048 > (size_t)h->max_smem) continue;
         Kernel64 kern = kernel_for(h->cfg, T);
         CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -626,20 +736,19 @@ int launch_forward64(swimmer_handle *h, const FwdArgs &a, int threads, int max_r
             continue;
         }
         if (fit < a.B) continue;
-        CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a, C));
+        CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a, C, 0));
         return 0;
     }
-    const int per = forward64_resident(h, threads);
+    const int per = forward64_resident(h, threads), pw = forward64_pair_warps(h, threads);
+    const size_t smem = forward64_smem(a.n_max, a.tab_panels, threads, pw);
     if (per < 1) {
-        set_error("forward kernel does not fit on an SM (threads %d, smem %zu)", threads,
-                  forward64_smem(a.n_max, a.tab_panels, threads));
+        set_error("forward kernel does not fit on an SM (threads %d, smem %zu)", threads, smem);
         return SWIMMER_E_CUDA;
     }
     // CTAs per SM: no more than the launch has runs per SM (see launch_forward)
     const int runs = max_runs > 0 && max_runs < a.B ? max_runs : a.B;
     const int per_sm = std::min(per, std::max(1, (runs + h->num_sms - 1) / h->num_sms));
-    kernel_for(h->cfg, threads)<<<std::min(per_sm * h->num_sms, a.B), threads,
-                                  forward64_smem(a.n_max, a.tab_panels, threads), s>>>(a, 1);
+    kernel_for(h->cfg, threads)<<<std::min(per_sm * h->num_sms, a.B), threads, smem, s>>>(a, 1, pw);
     CUDA_TRY(cudaGetLastError());
     return 0;
 }

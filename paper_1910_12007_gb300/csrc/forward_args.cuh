@@ -42,6 +42,7 @@ static __device__ __forceinline__ bool vel_obs(const FwdArgs &a, int nh) {
 
 // forward64.cu: dynamic shared memory of an FP64 launch and the launch itself (threads per CTA
 // as chosen by forward_threads)
-size_t forward64_smem(int n_max, int panels, int threads);
+size_t forward64_smem(int n_max, int panels, int threads, int pair_warps);
+int forward64_pair_warps(const swimmer_handle *h, int threads);
 int forward64_resident(const swimmer_handle *h, int threads);
 int launch_forward64(swimmer_handle *h, const FwdArgs &a, int threads, int max_runs, cudaStream_t s);
