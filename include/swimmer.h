@@ -147,7 +147,7 @@ int swimmer_kernel_eval(swimmer_handle *h, double alpha, double delta, double r_
  * memory (for example services whose device-memory budget is fixed at start-up, or code that
  * must not grow the process's allocations per request).  No
  * handle: the table build of the one sample runs on scratch held in file-scope device
- * arrays (about 0.2 MB, kept by every GPU that loads the library until the process exits).
+ * arrays (about 0.25 MB, kept by every GPU that loads the library until the process exits).
  * The paper has no counterpart; this is an interface convenience.
  *   - Same arguments and results as swimmer_kernel_eval; r, g1, g2 stay caller-owned.
  *   - Limit: r_max/delta < 4000 (24 octaves of u), alpha * r_max <= 600; larger sizes are

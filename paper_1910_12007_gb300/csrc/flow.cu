@@ -9,7 +9,8 @@
 // once per device in the same form) and the sources sit in shared memory, so a pair takes 16 FP64
 // instructions: separation and u 5, the three kernel functions one each, the sums 8.  With the
 // Clenshaw recurrences, square root and division in FP64 and the table read from L1 it took 75
-// (512 x 512 targets and 74 points: 2.8 ms a call, of it 2.75 here; now 0.65 ms a call).  CTAs are persistent: one or two per SM load the tables once and walk the targets.
+// (512 x 512 targets and 74 points: 2.8 ms a call, of it 2.75 here; now 0.65 ms a call).
+// CTAs are persistent: one or two per SM load the tables once and walk the targets.
 #include <math.h>
 #include <string.h>
 

@@ -157,6 +157,15 @@ __host__ __device__ size_t smem_bytes(int n_max, int P, int threads) {
     return state_bytes(n_max, threads) + table_bytes<MERGED>(P) + 4 * nbm * nbm;
 }
 
+// A run on a cluster: the state without partial velocities, the table as 32-byte records and, on a
+// 16-byte boundary after the units, every list's partial velocities of this step and of the next
+__host__ __device__ inline size_t cluster_part_at(int n_max, int P) {
+    return (smem_bytes<true>(n_max, P, 32) + 15) & ~size_t(15);
+}
+__host__ __device__ inline size_t cluster_smem(int n_max, int P, int list_threads) {
+    return cluster_part_at(n_max, P) + 2 * 256 * (size_t)((n_max + 31) / 32) * pair_warps(n_max, list_threads);
+}
+
 
 // -g1 and h = delta^2 g2 from the FP32 table: quadratic in G = 1 + f / 64, f in [0, 1) the
 // position of u within its panel.  The table holds -g1, the sign g1 takes in the mobility.
@@ -338,8 +347,18 @@ __device__ __forceinline__ void head_centre(const float *xh, const float *xl,
 // coupled by the fluid.  Code for models a launch does not run compiles out.  BIG: compiled
 // for at most 512 threads and one CTA per SM (up to 128 registers a thread), for launches
 // whose shared memory already holds them to that few threads per SM (large N): the pair
-// loop then keeps more loads in flight.
-template <int MODEL, bool BIG = false>
+// loop then keeps more loads in flight.  CLUSTER (with BIG): a run on a.cluster CTAs of a cluster, for
+// launches that leave SMs idle.  A run alone on an SM waits for its pair sum: at N = 128 the loads,
+// lookups and shuffles of its 16 units are about 3100 shared-memory wavefronts of a step's 7000 cycles.
+// The CTAs share out the lists of the sum; every CTA keeps the whole state and does all O(N) work itself,
+// the same operations on the same numbers, and a list's partial velocities go to all of them.  Two
+// buffers of these, by the step's parity, and one cluster barrier a step: who writes those of step s + 2
+// has passed the barrier of step s + 1, which every CTA reaches after it has read those of step s.  Measured,
+// us a step on one SM and on clusters of 2, 3 and 4: N = 128 3.38, 3.29, 3.01, 2.91; N = 192 6.51, 5.26, 4.87,
+// 4.66; N = 256 6.95, 5.61, 5.64, 5.21; N = 512 21.9, 14.3, 14.2, 12.0.  (Copies that arrive on an mbarrier
+// instead of the cluster barrier 3.00, 3.04, 2.96 at N = 128 and 4.54 on 4 at N = 192: as fast, and one
+// more wait to bound.)
+template <int MODEL, bool BIG = false, bool CLUSTER = false>
 __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a) {
     constexpr bool HEAD = MODEL >= 1, TWO = MODEL == 2;
     constexpr bool MERGED = BIG;  // the FP32 table as 32-byte records (see table_bytes)
@@ -355,7 +374,8 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
     R *tvy = tvx + n_max;
     R *bend = tvy + n_max;  // [6][n_max]
     float2 *part = (float2 *)tvx;  // FP32 pair sum: per-warp partial velocities
-    unsigned char *tabraw = smraw + state_bytes(n_max, blockDim.x);
+    unsigned char *tabraw = smraw + state_bytes(n_max, CLUSTER ? 32 : blockDim.x);
+    const int C = CLUSTER ? a.cluster : 1, rank = CLUSTER ? blockIdx.x % C : 0;
     __shared__ int s_work;
     // the sample's model constants: [0, 18) the springs (flagellum segment, head membrane,
     // diametral, neck A (end to H(pi +- dth)), neck B (next-to-end to H(pi +- dth)), neck
@@ -378,11 +398,17 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
     const int tid = threadIdx.x, T = blockDim.x;
     const int lane = tid & 31;
 
-    for (;;) {
-        if (tid == 0) s_work = atomicAdd(a.queue, 1);
-        __syncthreads();
-        const int w = s_work;
-        if (w >= a.B) break;
+    for (bool done = false;; done = true) {
+        int w;
+        if (CLUSTER) {  // a cluster per run
+            if (done) break;
+            w = blockIdx.x / C;
+        } else {
+            if (tid == 0) s_work = atomicAdd(a.queue, 1);
+            __syncthreads();
+            w = s_work;
+            if (w >= a.B) break;
+        }
         const int b = a.order[w];
         const SampleParams p = a.sp[b];
         const int nf = p.n, nh = HEAD ? p.nh : 0, h2 = nh >> 1;
@@ -390,13 +416,13 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
         const int n = TWO ? 2 * nsw : nsw;  // all points of the sample
         const long long n_obs = a.steps / a.obs_every;
         if (p.status != SWIMMER_OK) {
-            if (tid == 0) {
+            if (tid == 0 && rank == 0) {
                 a.status[b] = p.status;
                 if (a.loglik) a.loglik[b] = -INFINITY;
                 if (a.speed) a.speed[b] = nan("");
                 if (a.speculative) a.run_work[b] = 0;
             }
-            if (a.head_traj)
+            if (a.head_traj && rank == 0)
                 for (long long o = tid; o < 2 * n_obs; o += T) a.head_traj[(size_t)b * 2 * n_obs + o] = nan("");
             __syncthreads();
             continue;
@@ -517,7 +543,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
         // FP32 pair sum: the sample's units of 16 steps over the pair warps
         const unsigned *uhdr = a.units + a.mode * (UNIT_NB_MAX + 1);
         const int nb = (n + 31) >> 5, n_units = (int)(uhdr[nb] - uhdr[nb - 1]);
-        const int n_pw = min(pair_warps(n_max, T), (int)(uhdr[nbm] - uhdr[nbm - 1]));
+        const int n_pw = min(pair_warps(n_max, CLUSTER ? a.list_threads : T), (int)(uhdr[nbm] - uhdr[nbm - 1]));
         // the thread that keeps the log-likelihood: thread 0 for head-centre velocities (one
         // warp reduces the head after each observation step), else the one that updates the
         // proximal flagellum point nf - 1 (the observed point)
@@ -525,7 +551,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
         double J = 0.0;
         int status = SWIMMER_OK;
         long long steps_done = a.steps;
-        __syncthreads();
+        run_sync(C);  // (no CTA of a cluster writes to one that has not started)
         if (tid == 0)
             assign_units((unsigned *)(tabraw + table_bytes<MERGED>(P)), n_units, n_pw, (unsigned *)part, s_wstart);
         __syncthreads();
@@ -748,7 +774,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
             }
             __syncthreads();
             if (step == a.steps) {  // final state: positions and the forces there
-                for (int k = tid; k < n; k += T) {
+                for (int k = tid; k < n && rank == 0; k += T) {
                     double *o = a.final_state + ((size_t)b * n_max + k) * 4;
                     o[0] = ((double)xh[k] + (double)xl[k]) + xref;
                     o[1] = (double)yh[k] + (double)yl[k];
@@ -758,7 +784,9 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 break;
             }
             // ---- D: pair sum
-            if ((tid >> 5) < n_pw) {
+            if (CLUSTER) part = (float2 *)(smraw + cluster_part_at(n_max, P)) + ((step & 1) ? n_pw * (nb << 5) : 0);
+            const int list = CLUSTER ? (tid >> 5) * C + rank : tid >> 5;
+            if (list < n_pw) {
                 // FP32: each unordered pair {i, j} once.  g1(r) and g2(r) are even in
                 // d = X_i - X_j and (F . d) d is even too, so one table lookup gives both
                 // v_i += -F_j g1 + (F_j . d) d g2 and v_j += -F_i g1 + (F_i . d) d g2.
@@ -776,11 +804,10 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 const float4 *s4 = (const float4 *)src;
                 const float4 *tab = (const float4 *)tabraw;
                 const float2 *tB = (const float2 *)(tab + P);
-                const int warp = tid >> 5;
-                float2 *mypart = part + warp * (nb << 5);
+                float2 *mypart = part + list * (nb << 5);
                 for (int k = lane; k < (nb << 5); k += 32) mypart[k] = make_float2(0.f, 0.f);
                 const unsigned *units = (const unsigned *)(tabraw + table_bytes<MERGED>(P));
-                for (int un = s_wstart[warp]; un < s_wstart[warp + 1]; ++un) {
+                for (int un = s_wstart[list]; un < s_wstart[list + 1]; ++un) {
                     const unsigned pk = units[un];
                     const int I = pk & 31, Jb = (pk >> 5) & 31, code = (pk >> 25) & 3, kind = (pk >> 27) & 3;
                     const int d0 = code == 2 ? 1 : code << 4;
@@ -799,8 +826,19 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                         if (kind == 2) bad = 1;
                     }
                 }
+                if (CLUSTER) {  // to the other CTAs (a lane has summed what it sends)
+                    const unsigned at = smem_addr(mypart + lane);
+                    for (int r = rank + 1; r < rank + C; ++r) {
+                        const unsigned to = remote(at, r < C ? r : r - C);
+                        for (int q = 0; q < nb; ++q) {
+                            const float2 v = mypart[(q << 5) + lane];
+                            asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(to + 256 * q), "f"(v.x), "f"(v.y)
+                                         : "memory");
+                        }
+                    }
+                }
             }
-            __syncthreads();
+            run_sync(C);
             // ---- E: Euler step, divergence, observations
             for (int k = tid; k < n; k += T) {
                 // v_k = self term + the pair warps' partial sums, compensated
@@ -834,7 +872,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                             double rx = a.obs[2 * o] - hxo, ry = (a.obs[2 * o + 1] - hyo) / a.sigma_ratio;
                             J = fma(rx, rx, fma(ry, ry, J));
                         }
-                        if (a.head_traj) {
+                        if (a.head_traj && rank == 0) {
                             a.head_traj[((size_t)b * n_obs + o) * 2] = hxo;
                             a.head_traj[((size_t)b * n_obs + o) * 2 + 1] = hyo;
                         }
@@ -880,7 +918,7 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                         const double rx = a.obs[2 * o] - ox, ry = (a.obs[2 * o + 1] - oy) / a.sigma_ratio;
                         J = fma(rx, rx, fma(ry, ry, J));
                     }
-                    if (a.head_traj) {
+                    if (a.head_traj && rank == 0) {
                         a.head_traj[((size_t)b * n_obs + o) * 2] = ox;
                         a.head_traj[((size_t)b * n_obs + o) * 2 + 1] = oy;
                     }
@@ -890,6 +928,10 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 obs_left = obs_every;
                 ++obs_idx;
             }
+        }
+        if (CLUSTER) {
+            run_sync(C);  // every CTA stays until the others have written to it
+            if (rank != 0) break;
         }
         // ---- outputs
         if (a.final_state) {  // rows past the sample's points, or of a run that stopped: NaN
@@ -943,7 +985,18 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
     }
 }
 
+// Blocks of 32 points from which a run gains by a cluster, and the largest one that helps: us a step on one
+// SM and on clusters of 2, 4 and 8, N = 65 2.79, 2.75, 2.85, 3.4; N = 128 3.4, 3.3, 2.9, 3.4; N = 512 21.9, 14.3,
+// 12.0, 12.7 (every list goes to every CTA, so that the copies grow with the cluster).
+constexpr int CLUSTER_BLOCKS = 4, MAX_CLUSTER = 4;
+
 typedef void (*ForwardKernel)(FwdArgs);
+
+ForwardKernel cluster_kernel_for(const swimmer_config &c) {
+    return c.n_swimmers == 2 ? forward_kernel<2, true, true>
+           : c.n_head > 0    ? forward_kernel<1, true, true>
+                             : forward_kernel<0, true, true>;
+}
 
 ForwardKernel forward_kernel_for(const swimmer_config &c, bool big = false) {
     const int model = c.n_swimmers == 2 ? 2 : c.n_head > 0 ? 1 : 0;
@@ -1172,6 +1225,48 @@ int forward_threads(const swimmer_handle *h, int B, int precision) {
     return T;
 }
 
+// A launch that leaves half the SMs idle or more: every run on a cluster of the largest size that keeps
+// all runs on the device at once (at most a CTA a list).  The lists and their order are those of
+// the launch shape, so a run gives the same numbers as on one CTA.  done: whether it was launched.
+static int launch_cluster(swimmer_handle *h, FwdArgs &a, int list_threads, cudaStream_t s, bool &done) {
+    done = false;
+    const int nbm = (a.n_max + 31) / 32, lists = pair_warps(a.n_max, list_threads);
+    // (more than half of what an SM has: two CTAs on one SM would undo it)
+    const size_t smem = std::max(cluster_smem(a.n_max, a.tab_panels, list_threads), (size_t)h->max_smem / 2);
+    if (a.speculative || 2 * a.B > h->num_sms || nbm < CLUSTER_BLOCKS || smem + 1024 > (size_t)h->max_smem) return 0;
+    auto kern = cluster_kernel_for(h->cfg);
+    CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.dynamicSmemBytes = smem;
+    for (int C = std::min(MAX_CLUSTER, std::min(lists, h->num_sms / a.B)); C > 1; --C) {
+        const int need = 32 * ((lists + C - 1) / C);
+        int T = 256;
+        while (T < 512 && (T < need || T < a.n_max)) T <<= 1;
+        if (T < need) continue;
+        attr[0].val.clusterDim.x = C;
+        cfg.gridDim = dim3(a.B * C);
+        cfg.blockDim = dim3(T);
+        int fit = 0;
+        if (cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) != cudaSuccess) {
+            cudaGetLastError();  // a size that the device does not offer
+            continue;
+        }
+        if (fit < a.B) continue;
+        a.cluster = C;
+        a.list_threads = list_threads;
+        CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a));
+        done = true;
+        return 0;
+    }
+    return 0;
+}
+
 int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, double *loglik,
                    double *head_traj, double *mean_speed, int *status, int precision, cudaStream_t s,
                    int threads_override, int speculative, double *final_state, int max_runs) {
@@ -1270,8 +1365,13 @@ int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, do
     if (grid > B) grid = B;
     CUDA_TRY(cudaMemsetAsync(h->queue, 0, sizeof(int), s));
     prof_k2_begin(h, s, B);
-    kern<<<grid, T, smem, s>>>(a);
-    CUDA_TRY(cudaGetLastError());
+    bool done;
+    const int rc = launch_cluster(h, a, T, s, done);
+    if (rc) return rc;
+    if (!done) {
+        kern<<<grid, T, smem, s>>>(a);
+        CUDA_TRY(cudaGetLastError());
+    }
     prof_k2_end(h, s);
     prof_count(h, 1);
     return 0;

@@ -21,8 +21,9 @@
 // n / C points; forces and new positions go to every CTA's shared memory (double-buffered
 // positions, two cluster barriers a step).
 // Measured (whole calls): a lone run of N = 64, 2000 steps 53.1 -> 13.9 ms (26.5 -> 6.9 us a step) on a
-// cluster of 16; 1024 runs of N = 128, 200 steps 109 -> 99 ms; 152 pairs of sperm models (148
-// points), 400 steps 44 -> 40 ms.
+// cluster of 16; 1024 runs of N = 128, 200 steps 109 -> 65 ms (99 as a kernel of its own, 86 with 13
+// FP64 instructions a pair, 65 with the symmetric sum); 152 pairs of sperm models (148 points), 400
+// steps 44 -> 31.5 ms.
 #include <limits.h>
 #include <math.h>
 
@@ -54,12 +55,6 @@ __device__ __forceinline__ double spring(double2 xi, double2 xj, const Rest &r, 
     return r.k2 * strain * rs;
 }
 
-__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned remote(unsigned addr, unsigned rank) {
-    unsigned r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
 // a value at the same place of every CTA of the cluster
 __device__ __forceinline__ void put_all(double2 *p, double2 v, int C, int rank) {
     *p = v;
@@ -72,16 +67,6 @@ __device__ __forceinline__ void put_all(int *p, int v, int C, int rank) {
     for (int r = 0; r < C; ++r)
         if (r != rank)
             asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(smem_addr(p), r)), "r"(v) : "memory");
-}
-// barrier over the run's CTAs (every thread of every CTA reaches the same ones: all branches
-// around them depend on values that the CTAs share)
-__device__ __forceinline__ void run_sync(int C) {
-    if (C == 1) {
-        __syncthreads();
-    } else {
-        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    }
 }
 
 // shared memory before the table

@@ -32,12 +32,33 @@ struct FwdArgs {
     int tab_panels;  // panels of the shared-memory table region (handle's octaves x panels/octave)
     const unsigned *units;  // FP32 pair-unit lists (offsets header, then the lists)
     int mode;               // FP32 pair units: 0 one-, 1 two-, 2 four-target
+    int list_threads;       // FP32: the pair sum is split into as many lists as this many threads have warps
+    int cluster;            // FP32: CTAs per run
 };
 
 // observations computed by warp 0 after a step (head-centre velocities, two-swimmer
 // distances) rather than by the thread that updates the proximal point
 static __device__ __forceinline__ bool vel_obs(const FwdArgs &a, int nh) {
     return (a.obs_kind == SWIMMER_OBS_HEAD_VELOCITY || a.obs_kind == SWIMMER_OBS_PAIR_DISTANCES) && nh > 0;
+}
+
+// A run on a cluster of C CTAs: an address of this CTA's shared memory as that of the CTA of a rank, and
+// the barrier
+static __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+static __device__ __forceinline__ unsigned remote(unsigned addr, unsigned rank) {
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// barrier over the run's CTAs (every thread of every CTA reaches the same ones: all branches
+// around them depend on values that the CTAs share)
+static __device__ __forceinline__ void run_sync(int C) {
+    if (C == 1) {
+        __syncthreads();
+    } else {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    }
 }
 
 // forward64.cu: dynamic shared memory of an FP64 launch and the launch itself (threads per CTA

@@ -1291,7 +1291,8 @@ int launch_kernel_eval(swimmer_handle *h, int m, const double *r, double *g1, do
 // budget at start-up and must not grow it per request.  For them the
 // table build of one sample (the kernels above that use scratch memory) runs on scratch
 // that lives in file-scope device arrays: every GPU that loads this library holds these
-// ~0.2 MB until the process exits, and every call on a device shares them.
+// ~0.25 MB until the process exits, and every call on a device shares them (as handles do the
+// ~0.5 MB of universal nodes and quadrature points).
 namespace {
 __device__ __align__(256) double g_noalloc_scratch[K1_SCRATCH];
 __device__ __align__(256) float4 g_noalloc_tab64[TAB64_STRIDE];
