@@ -51,9 +51,9 @@ enum { SWIMMER_FP64 = 0, SWIMMER_FP32C = 1 };
 /* Launch-shape flags (FP32C only, at most one), OR-ed into a threads-per-sample value: the
  * pair sum takes two (WIDE) or four (QUAD) blocks of 32 targets per warp against one block of
  * sources, so each source load and shuffle serves two or four pair evaluations.  QUAD units
- * need 128 registers a thread: their launches hold at most 64K / 128 threads per SM (at most 512
- * threads a sample; beyond that, or where the 128-register kernel's table does not fit, WIDE
- * units run instead). */
+ * (from 225 points on; below, WIDE units run) need 128 registers a thread: their launches hold at
+ * most 64K / 128 threads per SM (at most 512 threads a sample; beyond that, or where the
+ * 128-register kernel's table does not fit, WIDE units run instead). */
 #define SWIMMER_SHAPE_WIDE 0x10000
 #define SWIMMER_SHAPE_QUAD 0x20000
 

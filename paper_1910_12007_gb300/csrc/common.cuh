@@ -47,6 +47,7 @@ constexpr int UNIT_HDR = UNIT_MODES * (UNIT_NB_MAX + 1);
 constexpr int SHAPE_WIDE = SWIMMER_SHAPE_WIDE;  // launch-shape flag: two-target pair units
 constexpr int SHAPE_QUAD = SWIMMER_SHAPE_QUAD;  // launch-shape flag: four-target pair units
 constexpr int SHAPE_THREADS = SHAPE_WIDE - 1;
+constexpr int SHAPE_WIDE128 = 0x40000;  // of the heuristic alone: two-target units at 128 registers a thread
 // unit packing: I [0, 5), J [5, 10), I2, I3, I4 [10, 25), step code [25, 27) (0: d0 = 0,
 // 1: d0 = 16, 2: diagonal block, d = 1 .. 16), kind [27, 29) (0, 1, 2: 1, 2, 4 target blocks)
 __host__ __device__ inline unsigned unit_pack(int kind, int code, int J, int I, int I2 = 0, int I3 = 0, int I4 = 0) {

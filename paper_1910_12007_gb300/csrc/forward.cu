@@ -1216,11 +1216,10 @@ int forward_threads(const swimmer_handle *h, int B, int precision) {
     while (T < cap && (long long)B * T * 2 <= (long long)h->num_sms * 1024 && forward_fits(h, 2 * T, precision))
         T <<= 1;
     // two-target units from 8 blocks of 32 points at every thread count, and from 4 blocks when the
-    // batch fills the GPU (the heuristic stays at 128 threads only then).  Below 8 blocks the four-target
-    // shape has the same lists; from six runs per SM on its four at a time at 128 registers beat five
-    // to seven at 64 (128 threads, 1100 runs: N = 128 14.6 against 16.0 us a step, N = 192 29.3, 32.3, N = 224
+    // batch fills the GPU (the heuristic stays at 128 threads only then).  From six
+    // runs per SM on, the same lists four at a time at 128 registers beat five to seven at 64 (128 threads, 1100 runs: N = 128 14.6 against 16.0 us a step, N = 192 29.3, 32.3, N = 224
     // 38.2, 42.4)
-    if (nbm >= 4 && nbm < 8 && T == 128 && bucket >= 5 && h->cfg.n_head == 0) return T | SHAPE_QUAD;
+    if (nbm >= 4 && nbm < 8 && T == 128 && bucket >= 5 && h->cfg.n_head == 0) return T | SHAPE_WIDE128;
     if (nbm >= 8 || (nbm >= 4 && T == 128)) return T | SHAPE_WIDE;
     return T;
 }
@@ -1310,7 +1309,7 @@ int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, do
     a.threads = T;
     const bool f64 = precision == SWIMMER_FP64;
     a.units = h->units;
-    a.mode = f64 ? 0 : (shape & SHAPE_QUAD) ? 2 : (shape & SHAPE_WIDE) ? 1 : 0;
+    a.mode = f64 ? 0 : (shape & SHAPE_QUAD) ? 2 : (shape & (SHAPE_WIDE | SHAPE_WIDE128)) ? 1 : 0;
     a.tab_panels = handle_octaves(h) * (f64 ? F64_FINE : F32_SUB);
     if (f64) {
         CUDA_TRY(cudaMemsetAsync(h->queue, 0, sizeof(int), s));
@@ -1337,10 +1336,11 @@ int launch_forward(swimmer_handle *h, int B, const double *obs, double sigma, do
     // FP32 with shared memory for so few threads per SM that each could hold 128 registers:
     // the instantiation compiled for that register budget (same CTAs per SM)
     // (with the table as 32-byte records, if that still fits)
-    // (four-target units are for that instantiation only: their launches hold fewer CTAs per SM
-    // when that many registers need it)
+    // (four-target units, which there are from 8 blocks on, are for that instantiation only: their
+    // launches hold fewer CTAs per SM when that many registers need it)
     const size_t smem_big = smem_bytes<true>(a.n_max, a.tab_panels, T);
-    if (a.mode == 2 && T <= 512 && smem_big + 1024 <= (size_t)h->max_smem)
+    const bool few_ctas = (a.mode == 2 && a.n_max > 7 * 32) || (shape & SHAPE_WIDE128);
+    if (few_ctas && T <= 512 && smem_big + 1024 <= (size_t)h->max_smem)
         per_sm = min(per_sm, max(1, h->regs_per_sm / (128 * T)));
     if (T <= 512 && per_sm >= 1 && (long long)per_sm * T * 128 <= h->regs_per_sm &&
         smem_big + 1024 <= (size_t)h->max_smem) {

@@ -143,6 +143,24 @@ def test_uneven_runs_on_clusters_equal_runs_on_one_sm(batch):
     h.close()
 
 
+@pytest.mark.parametrize("precision,batch", [(g.FP32C, 1), (g.FP32C, 40), (g.FP64, 1), (g.FP64, 30)])
+def test_cluster_launches_under_capture(precision, batch):
+    h = g.swimmer_init(g.SwimmerConfig(n_max=130, b_max=batch, dt=1e-8, steps=20, obs_every=5, precision=precision))
+    b = torch.arange(batch, dtype=torch.float64, device=DEV)
+    theta = torch.stack([0.5 + 0.02 * b, 0.1 * torch.sin(b), 0.09 + 0.01 * torch.cos(b)], 1).contiguous()
+    eager = g.forward_batch(h, theta)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = g.forward_batch(h, theta)
+    for _ in range(2):
+        out[0].zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, e) for a, e in zip(out, eager))
+    del graph
+    h.close()
+
+
 @pytest.mark.parametrize("alpha", [100.0, 300.0])
 def test_tables_of_strongly_screened_flow(alpha):
     # alpha delta up to 6, alpha r up to 570: intervals split in parts, products of large and small Bessel functions
