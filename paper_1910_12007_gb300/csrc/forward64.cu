@@ -168,6 +168,8 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
     unsigned rank_ = 0;
     if (C > 1) asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank_));
     const int rank = (int)rank_;
+    // every CTA of the cluster has started: only then may the others write to its shared memory
+    if (C > 1) run_sync(C);
 
     for (;;) {
         if (rank == 0 && tid == 0) put_all(&s_work, atomicAdd(a.queue, 1), C, 0);
