@@ -851,15 +851,15 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
                 }
                 float dx = (hx + lx) * s_f32[F_DTMU], dy = (hy + ly) * s_f32[F_DTMU];
                 if (!isfinite(dx) || !isfinite(dy) || fmaxf(fabsf(dx), fabsf(dy)) > s_f32[F_DS]) bad = 1;
-                float s, e, nh, nl;
+                float s, e, hi, lo;
                 two_sum(xh[k], dx, s, e);
-                two_sum(s, xl[k] + e, nh, nl);
-                xh[k] = nh;
-                xl[k] = nl;
+                two_sum(s, xl[k] + e, hi, lo);
+                xh[k] = hi;
+                xl[k] = lo;
                 two_sum(yh[k], dy, s, e);
-                two_sum(s, yl[k] + e, nh, nl);
-                yh[k] = nh;
-                yl[k] = nl;
+                two_sum(s, yl[k] + e, hi, lo);
+                yh[k] = hi;
+                yl[k] = lo;
                 // the head point's observation: squared residual into J (FP64), trajectory row;
                 // obs_step is the same for every thread, so other steps branch around it
                 if (obs_step) {
