@@ -215,8 +215,8 @@ int forward_batch_state(swimmer_handle *h, int B, const double *theta, const int
  * G_delta'(r)/r, d = x_g - X_j, from the n points of state (device [n][4] (x, y, F_x, F_y),
  * e.g. one sample of forward_batch_state) for the kernel of (alpha, delta).  grid: device
  * [G][2]; vel: device [G][2]; pres: device [G] (either may be NULL, not both).  r_max bounds
- * every target-to-point distance (the FP64 table is built to it; farther distances are
- * clamped).  Builds the table in the handle's sample slot 0.  Asynchronous on stream;
+ * every target-to-point distance of the velocity (its table is built to it; velocities of targets
+ * farther off mean nothing); the pressure holds at any distance.  Builds the table in the handle's sample slot 0.  Asynchronous on stream;
  * SWIMMER_E_ARG on bad sizes or parameters (alpha r_max beyond the table's reach gives NaN). */
 int swimmer_flow_field(swimmer_handle *h, double alpha, double delta, double r_max, int n, const double *state,
                        int G, const double *grid, double *vel, double *pres, void *stream);

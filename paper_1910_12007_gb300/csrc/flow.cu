@@ -33,6 +33,12 @@ constexpr int PRES_REC = 4;        // float4 per panel of the pressure kernel's 
 constexpr int PRES_PANELS = N_OCT_MAX * F64_FINE;
 __device__ float4 g_pressure[PRES_PANELS * PRES_REC];
 
+// delta^2 G_delta'(r)/r as a function of u: with q = u^(-1/2), q^2 (1 + q^2/(1 + q)) / (2 pi)
+__host__ __device__ __noinline__ double pressure_of_u(double u) {
+    const double q = 1.0 / sqrt(u);
+    return q * q * (1.0 + q * q / (1.0 + q)) / (2.0 * 3.14159265358979323846);
+}
+
 __global__ void __launch_bounds__(FLOW_THREADS) flow_kernel(int n, const double *__restrict__ state,
                                                             const float4 *__restrict__ tab64,
                                                             const SampleParams *__restrict__ sp, double mu, int G,
@@ -53,6 +59,8 @@ __global__ void __launch_bounds__(FLOW_THREADS) flow_kernel(int n, const double 
     if (pres)
         for (int i = threadIdx.x; i < panels * PRES_REC; i += FLOW_THREADS) ptab[i] = g_pressure[i];
     const double inv_d2 = 1.0 / (p.delta * p.delta), inv_mu = 1.0 / mu;
+    // high word of u at the tables' end (an FP64 comparison would cost a pair a sixteenth)
+    const unsigned u_end = 0x3ff00000u + ((unsigned)panels << (20 - F64_FINE_LOG2));
     const bool one_load = n <= FLOW_SOURCES;
     // every thread of the CTA takes the same number of turns (the barriers below)
     for (int g0 = blockIdx.x * FLOW_THREADS; g0 < G; g0 += gridDim.x * FLOW_THREADS) {
@@ -86,7 +94,10 @@ __global__ void __launch_bounds__(FLOW_THREADS) flow_kernel(int n, const double 
                     vx = fma(w, dx, vx);
                     vy = fma(w, dy, vy);
                 }
-                if (pres) pr = fma(fd, poly1_f64(ptab + PRES_REC * pan, th, tl), pr);
+                // (the pressure holds at any distance: beyond the octaves of r_max by its closed form)
+                if (pres)
+                    pr = fma(fd, (unsigned)__double2hiint(u) < u_end ? poly1_f64(ptab + PRES_REC * pan, th, tl)
+                                                                     : pressure_of_u(u), pr);
             }
         }
         if (g < G) {
@@ -97,12 +108,6 @@ __global__ void __launch_bounds__(FLOW_THREADS) flow_kernel(int n, const double 
             if (pres) pres[g] = pr * inv_d2;
         }
     }
-}
-
-// delta^2 G_delta'(r)/r as a function of u: with q = u^(-1/2), q^2 (1 + q^2/(1 + q)) / (2 pi)
-double pressure_of_u(double u) {
-    const double q = 1.0 / sqrt(u);
-    return q * q * (1.0 + q * q / (1.0 + q)) / (2.0 * 3.14159265358979323846);
 }
 
 }  // namespace
