@@ -3,13 +3,18 @@
 //
 // Bound by the FP64 pipe: GB300 issues a warp's FP64 instruction every 16 clocks of an SM, 64 times
 // slower than FP32.  So
-//   - positions are kept in units of delta (u = 1 + |e|^2 takes two FMAs), and the kernel functions
+//   - the pair sum reads positions in units of delta (u = 1 + |e|^2 takes two FMAs), and the kernel functions
 //     come from table_eval.cuh with one FP64 addition each: 13 FP64 instructions per ordered pair
 //     (separation 2, u 2, kernel functions 2, F . e and its product 3, the sums 4) where two
 //     Clenshaw recurrences took 54;
 //   - the threads that share a target leave their partial sums in shared memory and one thread adds
 //     them and updates the point: as warp shuffles, additions and the update cost their 16 clocks in
 //     every warp, for two or four useful lanes each;
+//   - a run's positions themselves are in the caller's units, and what rounding takes from one goes into
+//     its next displacement.  In units of delta their last place was up to 1.5 times coarser and the errors
+//     of all steps added up: against extended precision (400 steps, N = 64) positions were 1.4e-16 to
+//     2.9e-16 off in the mean square, now below 0.72e-16, and the forces at the end 1.7 to 6 times as far as
+//     now.  It costs a lone run 2 % of its time (N = 64, 2000 steps 13.9 -> 14.2 ms), a batch 0.3 %;
 //   - (cos, sin)(omega t) is made for 32 steps at a time, a lane each, and the preferred curvature
 //     is P_k cos + Q_k sin; springs and curvature take one reciprocal square root each.
 // Of a run that has a CTA to itself every unordered pair is evaluated once, in the blocks and units of
@@ -20,10 +25,10 @@
 // smooth filament they read the same table panel).  A lone run is spread over a cluster of up to 16 SMs: a CTA owns
 // n / C points; forces and new positions go to every CTA's shared memory (double-buffered
 // positions, two cluster barriers a step).
-// Measured (whole calls): a lone run of N = 64, 2000 steps 53.1 -> 13.9 ms (26.5 -> 6.9 us a step) on a
+// Measured (whole calls): a lone run of N = 64, 2000 steps 53.1 -> 14.2 ms (26.5 -> 7.1 us a step) on a
 // cluster of 16; 1024 runs of N = 128, 200 steps 109 -> 65 ms (99 as a kernel of its own, 86 with 13
 // FP64 instructions a pair, 65 with the symmetric sum); 152 pairs of sperm models (148 points), 400
-// steps 44 -> 31.5 ms.
+// steps 44 -> 31.6 ms.
 #include <limits.h>
 #include <math.h>
 
@@ -39,13 +44,12 @@ constexpr int MAX_CLUSTER = 16;
 constexpr int CLUSTER_THREADS = 256;  // threads of a CTA of a cluster (more when it owns more points)
 constexpr int CLUSTER_POINTS = 4;     // points of a CTA of a cluster at least
 
-// a Hookean spring E = K (l/l0 - 1)^2 l0 in units of delta: 1/l0^2, and 2 K delta / l0
+// a Hookean spring E = K (l/l0 - 1)^2 l0: 1/l0^2, and 2 K / l0
 struct Rest {
     double inv_l02, k2;
 };
 
-// t with force on i = t (X_j - X_i) (both in units of delta), and the strain l/l0 - 1 from
-// l^2/l0^2 - 1, without cancellation
+// t with force on i = t (X_j - X_i), and the strain l/l0 - 1 from l^2/l0^2 - 1, without cancellation
 __device__ __forceinline__ double spring(double2 xi, double2 xj, const Rest &r, double &ex, double &ey, double &strain) {
     ex = xj.x - xi.x;
     ey = xj.y - xi.y;
@@ -55,33 +59,58 @@ __device__ __forceinline__ double spring(double2 xi, double2 xj, const Rest &r, 
     return r.k2 * strain * rs;
 }
 
-// a value at the same place of every CTA of the cluster
-__device__ __forceinline__ void put_all(double2 *p, double2 v, int C, int rank) {
-    *p = v;
+// a value at the same place of every CTA of the cluster (its own among them: no branch in the loop;
+// C is even)
+__device__ __forceinline__ void put_all(double2 *p, double2 v, int C) {
+    if (C == 1) {
+        *p = v;
+        return;
+    }
+    const unsigned at = smem_addr(p);
+#pragma unroll 2
     for (int r = 0; r < C; ++r)
-        if (r != rank)
-            asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(remote(smem_addr(p), r)), "d"(v.x), "d"(v.y) : "memory");
+        asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(remote(at, r)), "d"(v.x), "d"(v.y) : "memory");
 }
-__device__ __forceinline__ void put_all(int *p, int v, int C, int rank) {
-    *p = v;
+__device__ __forceinline__ void put_all(double2 *p, double2 v, double2 *q, double2 w, int C) {
+    if (C == 1) {
+        *p = v;
+        *q = w;
+        return;
+    }
+    const unsigned at = smem_addr(p), off = smem_addr(q) - at;
+#pragma unroll 2
+    for (int r = 0; r < C; ++r) {
+        const unsigned to = remote(at, r);
+        asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(to), "d"(v.x), "d"(v.y) : "memory");
+        asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(to + off), "d"(w.x), "d"(w.y) : "memory");
+    }
+}
+__device__ __forceinline__ void put_all(int *p, int v, int C) {
+    if (C == 1) {
+        *p = v;
+        return;
+    }
     for (int r = 0; r < C; ++r)
-        if (r != rank)
-            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(smem_addr(p), r)), "r"(v) : "memory");
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(smem_addr(p), r)), "r"(v) : "memory");
 }
 
-// shared memory before the table
+// shared memory before the table (the pair sum's partial velocities lie over the stencils' terms, which the
+// force phase has read by then)
 __host__ __device__ inline size_t state_bytes(int n_max, int threads, int pair_warps) {
-    const size_t np = (n_max + 31) & ~31, part = pair_warps * np;
-    const size_t b = sizeof(double2) * (7 * np + (part > (size_t)threads ? part : (size_t)threads));
+    const size_t np = (n_max + 31) & ~31;
+    size_t part = pair_warps * np;
+    if (part < (size_t)threads) part = threads;
+    if (part < 3 * np) part = 3 * np;
+    const size_t b = sizeof(double2) * (5 * np + part);
     return (b + 127) & ~size_t(127);
 }
 
-// mean of the head points from k0 on (one warp, fixed order); all lanes get it
-__device__ __forceinline__ double2 centre(const double2 *pos, int k0, int count, int lane) {
+// mean of the points from k0 on as seen from ref (one warp, fixed order); all lanes get it
+__device__ __forceinline__ double2 centre(const double2 *P, double2 ref, int k0, int count, int lane) {
     double x = 0.0, y = 0.0;
     for (int m = lane; m < count; m += 32) {
-        x += pos[k0 + m].x;
-        y += pos[k0 + m].y;
+        x += P[k0 + m].x - ref.x;
+        y += P[k0 + m].y - ref.y;
     }
     for (int o = 16; o >= 1; o >>= 1) {
         x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -152,18 +181,21 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
     extern __shared__ __align__(128) unsigned char smraw[];
     const int n_max = a.n_max, T = blockDim.x, tid = threadIdx.x, lane = tid & 31;
     const int np = (n_max + 31) & ~31;     // points in blocks of 32
-    double2 *pos = (double2 *)smraw;       // [2][np] positions / delta, relative to (L/2, 0)
+    double2 *P = (double2 *)smraw;         // [np] positions relative to (L/2, 0)
+    double2 *pos = P + np;                 // [2][np] the same in units of delta, for the pair sum
     double2 *frc = pos + 2 * np;           // [np] point forces
-    double2 *tv = frc + np;                // [np] tension of segment (k, next)
+    double2 *pq = frc + np;                // [np] preferred-curvature coefficients
+    double2 *tv = pq + np;                 // [np] tension of segment (k, next)
     double2 *b0 = tv + np, *b4 = b0 + np;  // [np] bending of centre k on its neighbours
-    double2 *pq = b4 + np;                 // [np] preferred-curvature coefficients
-    double2 *part = pq + np;               // partial velocities: [T], or [pw][np] of the symmetric sum's warps
+    double2 *part = tv;                    // partial velocities: [T], or [pw][np] of the symmetric sum's warps
     const float4 *tab = (const float4 *)(smraw + state_bytes(n_max, T, pw));
     __shared__ int s_work, s_bad[2];
     __shared__ Rest s_rest[6];  // flagellum segment, head membrane, diametral, neck A, neck B, neck gap
-    // stencils of the flagellum [0] and the head [1]: delta/(2 h), delta/h^2, 1/(2 h), 1/h^2, 2 K h;
-    // then 1/H_r and 2 K_NA delta^3; the head centre at the previous observation
-    __shared__ double s_st[2][5], s_ihr, s_kang, s_c[2];
+    // stencils of the flagellum [0] and the head [1]: 1/(2 h), 1/h^2, 2 K h; then 1/H_r and 2 K_NA
+    __shared__ double s_st[2][3], s_ihr, s_kang;
+    // at the previous observation: the first head point and the head's centre as seen from there (a velocity
+    // is the difference of the large parts, which is exact, and of the small ones)
+    __shared__ double2 s_first, s_centre;
     __shared__ double2 s_rot[32];  // (cos, sin)(omega t) of 32 steps
     unsigned rank_ = 0;
     if (C > 1) asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank_));
@@ -172,7 +204,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
     if (C > 1) run_sync(C);
 
     for (;;) {
-        if (rank == 0 && tid == 0) put_all(&s_work, atomicAdd(a.queue, 1), C, 0);
+        if (rank == 0 && tid == 0) put_all(&s_work, atomicAdd(a.queue, 1), C);
         run_sync(C);
         const int w = s_work;
         if (w >= a.B) break;
@@ -221,6 +253,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                 y0 = hr * sn;
             }
             if (sw) y0 += a.swim_d;
+            P[k] = make_double2(x0, y0);
             pos[k] = make_double2(x0 * inv_d, y0 * inv_d);
             if (kl < nf) {
                 // the preferred curvature (Appendix: y^ = a (1 - s/L) sin(eta s - omega t),
@@ -248,19 +281,17 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
             const double kk[6] = {a.kt, a.k_head_tens, a.k_head_tens, a.k_neck_tens, a.k_neck_tens, a.k_neck_tens};
             for (int q = 0; q < 6; ++q) {
                 const double lq = l0[q] > 0.0 ? l0[q] : 1.0;  // unused without a head
-                s_rest[q].inv_l02 = delta * delta / (lq * lq);
-                s_rest[q].k2 = 2.0 * kk[q] * delta / lq;
+                s_rest[q].inv_l02 = 1.0 / (lq * lq);
+                s_rest[q].k2 = 2.0 * kk[q] / lq;
             }
             for (int q = 0; q < (nh ? 2 : 1); ++q) {
                 const double h = q ? dsh : ds;
-                s_st[q][0] = 0.5 * delta / h;
-                s_st[q][1] = delta / (h * h);
-                s_st[q][2] = 0.5 / h;
-                s_st[q][3] = 1.0 / (h * h);
-                s_st[q][4] = 2.0 * (q ? a.k_head_c : p.kc) * h;
+                s_st[q][0] = 0.5 / h;
+                s_st[q][1] = 1.0 / (h * h);
+                s_st[q][2] = 2.0 * (q ? a.k_head_c : p.kc) * h;
             }
             s_ihr = nh ? 1.0 / hr : 0.0;
-            s_kang = 2.0 * a.k_neck_ang * delta * delta * delta;
+            s_kang = 2.0 * a.k_neck_ang;
             s_bad[0] = s_bad[1] = 0;
         }
         // the CTA's own points, and the threads of the pair sum: thread -> (own point, split)
@@ -270,7 +301,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
         // lanes that add a point's partial sums: eight for a few points, else one
         const int G = m < 32 && 8 * m <= T ? 8 : 1;
         const int my = G == 8 ? tid >> 3 : tid;  // own point that this thread updates (if < m)
-        const double dt_c = a.dt / (a.mu * delta), ds_d = ds * inv_d;
+        const double dt_mu = a.dt / a.mu;
         const double self_g1 = [&] {
             __syncthreads();
             double g1, h;
@@ -282,14 +313,15 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
         const bool vobs = vel_obs(a, nh);
         const bool head_thread = vobs ? rank == 0 && tid == 0
                                       : my == nf - 1 - k_lo && my < m && (G == 1 || (tid & 7) == 0);
+        double2 rest = make_double2(0.0, 0.0);  // what rounding took from the position that this thread updates
         double J = 0.0;
         int status = SWIMMER_OK;
         long long steps_done = a.steps;
         if (vobs && rank == 0 && tid < 32) {  // head centre at the previous observation
-            const double2 c = centre(pos, nf, nh, lane);
+            const double2 c = centre(P, P[nf], nf, nh, lane);
             if (tid == 0) {
-                s_c[0] = c.x;
-                s_c[1] = c.y;
+                s_first = P[nf];
+                s_centre = c;
             }
         }
         run_sync(C);
@@ -335,17 +367,17 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                 const int next = hd ? base + nf + (mh + 1 == nh ? 0 : mh + 1) : (kl + 1 < nf ? k + 1 : -1);
                 const int prev = hd ? base + nf + (mh == 0 ? nh - 1 : mh - 1) : k - 1;
                 const bool center = hd || (kl >= 1 && kl + 1 < nf);
-                const double2 xk = X[k];
+                const double2 xk = P[k];
                 double epx = 0.0, epy = 0.0;
                 if (next >= 0) {
                     double strain;
-                    const double t = spring(xk, X[next], s_rest[hd ? 1 : 0], epx, epy, strain);
+                    const double t = spring(xk, P[next], s_rest[hd ? 1 : 0], epx, epy, strain);
                     if (!(fabs(strain) <= STRETCH_MAX)) bad = 1;
                     tv[k] = make_double2(t * epx, t * epy);
                 }
                 if (center) {
                     const double *st = s_st[hd ? 1 : 0];
-                    const double emx = xk.x - X[prev].x, emy = xk.y - X[prev].y;
+                    const double emx = xk.x - P[prev].x, emy = xk.y - P[prev].y;
                     const double A = (emx + epx) * st[0], Bv = (emy + epy) * st[0];
                     const double Cc = (epx - emx) * st[1], D = (epy - emy) * st[1];
                     const double rs = rsqrt(fma(A, A, Bv * Bv)), r2 = rs * rs, S15 = r2 * rs;
@@ -355,7 +387,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                         const double2 c = pq[k], rot = s_rot[step & 31];
                         zhat = fma(c.x, rot.x, c.y * rot.y);
                     }
-                    const double ck = st[4] * (zeta - zhat), p1 = ck * st[2], p2 = ck * st[3] * S15;
+                    const double ck = st[2] * (zeta - zhat), p1 = ck * st[0], p2 = ck * st[1] * S15;
                     const double s25 = 3.0 * zeta * r2;
                     const double Px = fma(D, S15, -A * s25) * p1, Py = -fma(Cc, S15, Bv * s25) * p1;
                     const double Qx = -Bv * p2, Qy = A * p2;
@@ -419,7 +451,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                         }
                         if (j < 0) continue;
                         double ex, ey, strain;
-                        const double t = spring(X[k], X[j + base], s_rest[2 + kind], ex, ey, strain);
+                        const double t = spring(P[k], P[j + base], s_rest[2 + kind], ex, ey, strain);
                         fx += t * ex;
                         fy += t * ey;
                         if (!(fabs(strain) <= STRETCH_MAX)) bad = 1;
@@ -427,8 +459,8 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                     // neck angle E = K (z1 . z2)^2, z1 = H(pi) - X_{nf-1}, z2 = H(pi+dth) - H(pi-dth)
                     const int ihp = base + nf + h2, iplus = ihp + 1, iminus = ihp - 1, iend = base + nf - 1;
                     if (k == ihp || k == iplus || k == iminus || k == iend) {
-                        const double z1x = X[ihp].x - X[iend].x, z1y = X[ihp].y - X[iend].y;
-                        const double z2x = X[iplus].x - X[iminus].x, z2y = X[iplus].y - X[iminus].y;
+                        const double z1x = P[ihp].x - P[iend].x, z1y = P[ihp].y - P[iend].y;
+                        const double z2x = P[iplus].x - P[iminus].x, z2y = P[iplus].y - P[iminus].y;
                         const double ww = s_kang * (z1x * z2x + z1y * z2y);
                         if (k == ihp) {
                             fx -= ww * z2x;
@@ -445,15 +477,15 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                         }
                     }
                 }
-                put_all(frc + k, make_double2(fx, fy), C, rank);
+                put_all(frc + k, make_double2(fx, fy), C);
             }
             run_sync(C);
             if (step == a.steps) {  // final state: positions and the forces there
                 for (int q = tid; q < m; q += T) {
                     const int k = k_lo + q;
                     double *o = a.final_state + ((size_t)b * n_max + k) * 4;
-                    o[0] = fma(X[k].x, delta, xref);
-                    o[1] = X[k].y * delta;
+                    o[0] = P[k].x + xref;
+                    o[1] = P[k].y;
                     o[2] = frc[k].x;
                     o[3] = frc[k].y;
                 }
@@ -538,16 +570,18 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                 }
             }
             // ---- E: Euler step into the other position buffer, divergence, observations
-            double2 *Xn = pos + ((step + 1) & 1) * np;
             if (my < m && (G == 1 || (tid & 7) == 0)) {
                 const int k = k_lo + my;
-                const double dx = vx * dt_c, dy = vy * dt_c;  // displacement this step
-                if (!isfinite(dx) || !isfinite(dy) || fmax(fabs(dx), fabs(dy)) > ds_d) bad = 1;
-                const double2 xn = make_double2(X[k].x + dx, X[k].y + dy);
-                put_all(Xn + k, xn, C, rank);
+                // the displacement with what the last sum left over
+                const double2 was = P[k];
+                const double2 moved = make_double2(fma(vx, dt_mu, rest.x), fma(vy, dt_mu, rest.y));
+                if (!isfinite(moved.x) || !isfinite(moved.y) || fmax(fabs(moved.x), fabs(moved.y)) > ds) bad = 1;
+                const double2 xn = make_double2(was.x + moved.x, was.y + moved.y);
+                put_all(pos + ((step + 1) & 1) * np + k, make_double2(xn.x * inv_d, xn.y * inv_d), P + k, xn, C);
+                rest = make_double2(moved.x - (xn.x - was.x), moved.y - (xn.y - was.y));
                 // the head point's observation: squared residual into J, trajectory row
                 if (obs_step && !vobs && k == nf - 1) {
-                    const double hxo = fma(xn.x, delta, xref), hyo = xn.y * delta;
+                    const double hxo = xn.x + xref, hyo = xn.y;
                     const long long o = obs_idx;
                     if (a.obs) {
                         const double rx = a.obs[2 * o] - hxo, ry = (a.obs[2 * o + 1] - hyo) / a.sigma_ratio;
@@ -560,7 +594,7 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                 }
             }
             // (two flags in turn: a CTA ahead in the next step must not be read here)
-            if (bad) put_all(&s_bad[step & 1], 1, C, rank);
+            if (bad) put_all(&s_bad[step & 1], 1, C);
             run_sync(C);
             if (s_bad[step & 1]) {
                 status = SWIMMER_DIVERGED;
@@ -571,20 +605,22 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
                 double ox, oy;
                 if (TWO && a.obs_kind == SWIMMER_OBS_PAIR_DISTANCES) {
                     // distances between the tail tips and between the head centres (Sec. 4.2)
-                    const double2 c0 = centre(Xn, nf, nh, lane), c1 = centre(Xn, nsw + nf, nh, lane);
-                    const double tx = Xn[nsw].x - Xn[0].x, ty = Xn[nsw].y - Xn[0].y;
-                    ox = sqrt(tx * tx + ty * ty) * delta;
-                    oy = sqrt((c1.x - c0.x) * (c1.x - c0.x) + (c1.y - c0.y) * (c1.y - c0.y)) * delta;
+                    const double2 f0 = P[nf], f1 = P[nsw + nf];
+                    const double2 c0 = centre(P, f0, nf, nh, lane), c1 = centre(P, f1, nsw + nf, nh, lane);
+                    const double cx = (f1.x - f0.x) + (c1.x - c0.x), cy = (f1.y - f0.y) + (c1.y - c0.y);
+                    const double tx = P[nsw].x - P[0].x, ty = P[nsw].y - P[0].y;
+                    ox = sqrt(tx * tx + ty * ty);
+                    oy = sqrt(cx * cx + cy * cy);
                 } else {
                     // head-centre velocity over the observation interval (Sec. 4.1)
-                    const double2 c = centre(Xn, nf, nh, lane);
-                    const double inv = delta / ((double)a.obs_every * a.dt);
-                    ox = (c.x - s_c[0]) * inv;
-                    oy = (c.y - s_c[1]) * inv;
+                    const double2 f = P[nf], c = centre(P, f, nf, nh, lane);
+                    const double inv = 1.0 / ((double)a.obs_every * a.dt);
+                    ox = ((f.x - s_first.x) + (c.x - s_centre.x)) * inv;
+                    oy = ((f.y - s_first.y) + (c.y - s_centre.y)) * inv;
                     __syncwarp();
                     if (tid == 0) {
-                        s_c[0] = c.x;
-                        s_c[1] = c.y;
+                        s_first = f;
+                        s_centre = c;
                     }
                 }
                 if (tid == 0) {
@@ -615,10 +651,10 @@ __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, in
             // coordinates) or, with a head, of the head centre (the first swimmer's, with two), over
             // the run's duration; one warp sums in a fixed order
             const int k0 = nh > 0 ? nf : 0;
-            const double2 c = centre(pos + (a.steps & 1) * np, k0, nsw - k0, lane);
+            const double2 ref = nh > 0 ? P[k0] : make_double2(0.0, 0.0), c = centre(P, ref, k0, nsw - k0, lane);
             if (tid == 0) {
                 const double c0 = nh > 0 ? L + (a.gap_over_ds + a.hr_over_ds) * ds - xref : 0.0;
-                a.speed[b] = status == SWIMMER_OK ? (c.x * delta - c0) / (a.steps * a.dt) : nan("");
+                a.speed[b] = status == SWIMMER_OK ? ((ref.x - c0) + c.x) / (a.steps * a.dt) : nan("");
             }
         }
         if (rank == 0 && tid == 0) {
