@@ -204,8 +204,8 @@ int swimmer_tuning(swimmer_handle *h, int precision, int *threads, int set);
 
 /* forward_batch that also returns each run's final state: final_state (device
  * [B][n_max][4] FP64) = (x, y, F_x, F_y) of every point at t = steps dt, the forces
- * recomputed there (Eq. Fenergy); rows past a sample's points and runs that stopped early are
- * NaN.  Points: flagellum 0..n-1, then the head, then the second swimmer's.  Used for the
+ * recomputed there (Eq. Fenergy); rows past a sample's points, runs that stopped early and samples
+ * outside the domain are NaN.  Points: flagellum 0..n-1, then the head, then the second swimmer's.  Used for the
  * flow field below.  Errors as forward_batch. */
 int forward_batch_state(swimmer_handle *h, int B, const double *theta, const int *n_pts, double *head_traj,
                         double *mean_speed, int *status, double *final_state, void *stream);

@@ -424,6 +424,8 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
             }
             if (a.head_traj && rank == 0)
                 for (long long o = tid; o < 2 * n_obs; o += T) a.head_traj[(size_t)b * 2 * n_obs + o] = nan("");
+            if (a.final_state && rank == 0)
+                for (int k = tid; k < 4 * n_max; k += T) a.final_state[(size_t)b * 4 * n_max + k] = nan("");
             __syncthreads();
             continue;
         }
