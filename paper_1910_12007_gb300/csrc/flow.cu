@@ -10,6 +10,9 @@
 // instructions: separation and u 5, the three kernel functions one each, the sums 8.  With the
 // Clenshaw recurrences, square root and division in FP64 and the table read from L1 it took 75
 // (512 x 512 targets and 74 points: 2.8 ms a call, of it 2.75 here; now 0.65 ms a call).
+// Against extended precision (30 points) the pressure is 3.6e-17 of its terms' sizes off in the mean square and the
+// velocity 8.2e-17, where the closed form and the recurrences in FP64 were 4.4e-17 and 15e-17; with the
+// pressure's table fitted in FP64 it had been 17e-17.
 // CTAs are persistent: one or two per SM load the tables once and walk the targets.
 #include <math.h>
 #include <string.h>
@@ -23,7 +26,7 @@
 
 int launch_set_sample(swimmer_handle *h, double alpha, double delta, double r_max, cudaStream_t s);
 int launch_table_build(swimmer_handle *h, int B, int need64, cudaStream_t s);
-void fit_powers(int n, int deg, double (*f)(double), double lo, double hi, double *c);
+void fit_matrix(int n, int deg, long double *node, long double *weight);
 
 namespace {
 
@@ -33,10 +36,15 @@ constexpr int PRES_REC = 4;        // float4 per panel of the pressure kernel's 
 constexpr int PRES_PANELS = N_OCT_MAX * F64_FINE;
 __device__ float4 g_pressure[PRES_PANELS * PRES_REC];
 
-// delta^2 G_delta'(r)/r as a function of u: with q = u^(-1/2), q^2 (1 + q^2/(1 + q)) / (2 pi)
-__host__ __device__ __noinline__ double pressure_of_u(double u) {
+// delta^2 G_delta'(r)/r as a function of u: with q = u^(-1/2), q^2 (1 + q^2/(1 + q)) / (2 pi); on the
+// host, for the table's fit, in extended precision
+__device__ __noinline__ double pressure_of_u(double u) {
     const double q = 1.0 / sqrt(u);
     return q * q * (1.0 + q * q / (1.0 + q)) / (2.0 * 3.14159265358979323846);
+}
+long double pressure_to_fit(long double u) {
+    const long double q = 1.0L / sqrtl(u);
+    return q * q * (1.0L + q * q / (1.0L + q)) / (2.0L * acosl(-1.0L));
 }
 
 __global__ void __launch_bounds__(FLOW_THREADS) flow_kernel(int n, const double *__restrict__ state,
@@ -122,17 +130,24 @@ int pressure_init() {
     ARG_CHECK(dev >= 0 && dev < 256, "device ordinal %d out of range", dev);
     if (done[dev]) return 0;
     std::vector<float4> all(PRES_PANELS * PRES_REC);
+    constexpr int NODES = 10, COEFS = 8;
+    long double node[NODES], weight[COEFS][NODES];
+    fit_matrix(NODES, COEFS - 1, node, weight[0]);
     for (int q = 0; q < PRES_PANELS; ++q) {
         const double oct = ldexp(1.0, q / F64_FINE), w = oct / F64_FINE, lo = oct + (q % F64_FINE) * w;
-        double c[8];
-        fit_powers(10, 7, pressure_of_u, lo, lo + w, c);
+        long double c[COEFS] = {};
+        for (int i = 0; i < NODES; ++i) {
+            const long double v = pressure_to_fit(lo + 0.5L * w * (node[i] + 1.0L));
+            for (int k = 0; k < COEFS; ++k) c[k] += weight[k][i] * v;
+        }
         float h[6], l[6];
         for (int k = 1; k <= 5; ++k) {
             h[k] = (float)c[k];
-            l[k] = (float)(c[k] - (double)h[k]);
+            l[k] = (float)(c[k] - (long double)h[k]);
         }
         float4 *rec = &all[q * PRES_REC];
-        memcpy(rec, c, sizeof(double));
+        const double c0 = (double)c[0];
+        memcpy(rec, &c0, sizeof(double));
         rec[0].z = h[1];
         rec[0].w = l[1];
         rec[1] = make_float4(h[5], l[5], h[4], l[4]);

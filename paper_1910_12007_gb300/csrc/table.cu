@@ -1000,12 +1000,13 @@ static double host_i_scaled(int nu, double x) {
 }
 
 // Chebyshev coefficients in [-1, 1] to powers (in place, n of them)
-static void cheb_to_powers(double *c, int n) {
-    std::vector<double> out(n, 0.0), t0(n, 0.0), t1(n, 0.0), t2(n, 0.0);
+template <class T>
+static void cheb_to_powers(T *c, int n) {
+    std::vector<T> out(n, 0.0), t0(n, 0.0), t1(n, 0.0), t2(n, 0.0);
     t0[0] = 1.0;
     if (n > 1) t1[1] = 1.0;
     for (int k = 0; k < n; ++k) {
-        const std::vector<double> &tk = k == 0 ? t0 : t1;
+        const std::vector<T> &tk = k == 0 ? t0 : t1;
         for (int i = 0; i < n; ++i) out[i] += c[k] * tk[i];
         if (k >= 1) {
             for (int i = 0; i < n; ++i) t2[i] = (i ? 2.0 * t1[i - 1] : 0.0) - t0[i];
@@ -1015,17 +1016,19 @@ static void cheb_to_powers(double *c, int n) {
     }
     std::copy(out.begin(), out.end(), c);
 }
-// powers of t, t in [-1, 1] across [lo, hi], of f's polynomial through n Chebyshev nodes cut to
-// degree deg (its Chebyshev series, so that what is cut is small)
-void fit_powers(int n, int deg, double (*f)(double), double lo, double hi, double *c) {
-    std::vector<double> v(n);
-    for (int i = 0; i < n; ++i) v[i] = f(lo + 0.5 * (hi - lo) * (cos(PI * (i + 0.5) / n) + 1.0));
-    for (int k = 0; k <= deg; ++k) {
-        double s = 0.0;
-        for (int i = 0; i < n; ++i) s += v[i] * cos(PI * k * (i + 0.5) / n);
-        c[k] = s * (k == 0 ? 1.0 : 2.0) / n;
+// The fit of a function on [-1, 1] in powers of t: its polynomial through n Chebyshev nodes as a Chebyshev
+// series cut to degree deg (so that what is cut is small).  node [n]; weight [deg + 1][n] takes the values there
+// to the coefficients.  In extended precision: rounding of these sums would show in the leading coefficient's
+// last places.
+void fit_matrix(int n, int deg, long double *node, long double *weight) {
+    const long double pi = acosl(-1.0L);
+    for (int i = 0; i < n; ++i) {
+        node[i] = cosl(pi * (i + 0.5L) / n);
+        std::vector<long double> c(deg + 1);
+        for (int k = 0; k <= deg; ++k) c[k] = cosl(pi * k * (i + 0.5L) / n) * (k == 0 ? 1.0L : 2.0L) / n;
+        cheb_to_powers(c.data(), deg + 1);
+        for (int k = 0; k <= deg; ++k) weight[k * n + i] = c[k];
     }
-    cheb_to_powers(c, deg + 1);
 }
 
 // powers of t = z_scale z + z_shift of f(1/z) on x in [lo, 1/inv_hi], degree deg
