@@ -28,8 +28,7 @@
 //      one unit (each source load and rotation then serves two or four targets per lane);
 //      the host builds the unit lists per block count.  Per-warp partial sums are combined
 //      in a fixed order with TwoSum, so results do not depend on scheduling.  Launches
-//      whose shared memory holds an SM to one CTA of at most 512 threads use an
-//      instantiation compiled for 128 registers a thread.
+//      that hold an SM to 16 warps use an instantiation compiled for 128 registers a thread.
 //   E  forward Euler X += dt v: double-float (hi + lo FP32, about 48 significant bits)
 //      positions updated by TwoSum;
 //      every obs_every steps the head point is compared with the observations and the
@@ -115,8 +114,8 @@ __device__ __forceinline__ float spring_f32(const float *xh, const float *xl, co
 
 // table region in shared memory: float4 part A [P] then float2 part B [P] (24 bytes a
 // panel), or with MERGED one 32-byte record per panel [P][2] float4, so that one address serves
-// both loads of a lookup (the 128-register instantiation, whose launches are held to one or two
-// CTAs per SM by other limits, so the larger table costs no occupancy there);
+// both loads of a lookup (the 128-register instantiation, whose launches hold at most 16 warps an SM, so that
+// the larger table seldom costs a CTA)
 template <bool MERGED = false>
 __host__ __device__ size_t table_bytes(int P) {
     return (MERGED ? 2 * sizeof(float4) : sizeof(float4) + sizeof(float2)) * P;
@@ -345,8 +344,8 @@ __device__ __forceinline__ void head_centre(const float *xh, const float *xl,
 
 // MODEL 0: the flagellum; 1: the full sperm model (head points and neck); 2: two sperm models
 // coupled by the fluid.  Code for models a launch does not run compiles out.  BIG: compiled
-// for at most 512 threads and one CTA per SM (up to 128 registers a thread), for launches
-// whose shared memory already holds them to that few threads per SM (large N): the pair
+// for at most 512 threads at up to 128 registers each, for launches of 16 warps an SM (one CTA of 512
+// threads up to four of 128), which shared memory or the launch shape holds to that few: the pair
 // loop then keeps more loads in flight.  CLUSTER (with BIG): a run on a.cluster CTAs of a cluster, for
 // launches that leave SMs idle.  A run alone on an SM waits for its pair sum: at N = 128 the loads,
 // lookups and shuffles of its 16 units are about 3100 shared-memory wavefronts of a step's 7000 cycles.
@@ -989,7 +988,9 @@ __global__ void __launch_bounds__(BIG ? 512 : 1024, 1) forward_kernel(FwdArgs a)
 
 // Blocks of 32 points from which a run gains by a cluster, and the largest one that helps: us a step on one
 // SM and on clusters of 2, 4 and 8, N = 65 2.79, 2.75, 2.85, 3.4; N = 128 3.4, 3.3, 2.9, 3.4; N = 512 21.9, 14.3,
-// 12.0, 12.7 (every list goes to every CTA, so that the copies grow with the cluster).
+// 12.0, 12.7 (every list goes to every CTA, so that the copies grow with the cluster).  Either side of the line, on
+// one SM and on the cluster that the launch would take: three blocks, N = 65 2.67, 2.69 (one run), 2.76, 2.61 (40
+// runs), N = 96 2.61, 2.67 and 2.68, 2.58; four blocks, N = 97 3.29, 2.81 and 3.42, 2.98.
 constexpr int CLUSTER_BLOCKS = 4, MAX_CLUSTER = 4;
 
 typedef void (*ForwardKernel)(FwdArgs);
@@ -1200,7 +1201,11 @@ int forward_threads(const swimmer_handle *h, int B, int precision) {
     // from about 700 points two runs' shared memory no longer fits: N = 768 512q 49.7, 99.3, 198, 256q
     // 53.2, 106, 212.  (Two-target units and as many threads as the batch leaves: N = 512 31.4, 52.7,
     // 92.5, 236.)  Below, where a shorter step's larger displacements show the order of the pair sum in
-    // a log-likelihood's ninth digit, shapes keep their partition of the sum.
+    // a log-likelihood's ninth digit, shapes keep their partition of the sum.  So do head models of any size: an
+    // observed head velocity is a small difference of positions, and with four-target units it moves by 1e-5 to
+    // 3e-5 of the largest (300 points), which a user would see; what they would save is less (us a step of
+    // 100, 300 and 1100 runs, as here and with the better of 512q and 256q: 300 points 15.3, 27.1, 142 and 13.6,
+    // 24.9, 141; 540 points, 100 and 300 runs, 36.5, 80.1 and 33.2, 68.2).  An autotuned handle takes them.
     if (h->cfg.n_head == 0 && nbm >= 8) {
         int shape;
         if (bucket == 0) {
@@ -1218,9 +1223,11 @@ int forward_threads(const swimmer_handle *h, int B, int precision) {
     while (T < cap && (long long)B * T * 2 <= (long long)h->num_sms * 1024 && forward_fits(h, 2 * T, precision))
         T <<= 1;
     // two-target units from 8 blocks of 32 points at every thread count, and from 4 blocks when the
-    // batch fills the GPU (the heuristic stays at 128 threads only then).  From six
-    // runs per SM on, the same lists four at a time at 128 registers beat five to seven at 64 (128 threads, 1100 runs: N = 128 14.6 against 16.0 us a step, N = 192 29.3, 32.3, N = 224
-    // 38.2, 42.4)
+    // batch fills the GPU (the heuristic stays at 128 threads only then).  From six runs per SM on, the
+    // same lists four CTAs at a time at 128 registers beat five to seven at 64, with the same bits (128
+    // threads, 1100 runs: N = 128 14.6 against 16.0 us a step, N = 192 29.3, 32.3, N = 224 38.2, 42.4).  Tuning
+    // tables do not name that form: the autotuner's draws stop early more often than a stage's runs and
+    // would choose it where it loses.
     if (nbm >= 4 && nbm < 8 && T == 128 && bucket >= 5 && h->cfg.n_head == 0) return T | SHAPE_WIDE128;
     if (nbm >= 8 || (nbm >= 4 && T == 128)) return T | SHAPE_WIDE;
     return T;

@@ -174,7 +174,9 @@ __host__ __device__ inline bool symmetric_pays(int n) {
 }
 
 // MODEL 0: the flagellum; 1: the full sperm model (head points and neck); 2: two sperm models
-// coupled by the fluid.  C CTAs (a cluster when C > 1) share a run.
+// coupled by the fluid.  MAXT 1024, for runs above 512 points, is held to 64 registers and spills (360 to 560
+// bytes of loads a thread): 100 runs take, us a step, N = 600 2000, N = 768 4530, N = 1024 7400, a fifth to a
+// quarter of what the Clenshaw kernel took (10500, 16700, 29100).  C CTAs (a cluster when C > 1) share a run.
 template <int MODEL, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, int pw) {
     constexpr bool HEAD = MODEL >= 1, TWO = MODEL == 2;

@@ -6,9 +6,10 @@
 // Panels: 32 per octave of u = 1 + r^2/delta^2, indexed by the double's exponent and top 5
 // mantissa bits; t in [-1, 1) across a panel is the remaining 47 bits, split exactly into two
 // floats th + tl by integer operations.  On so short a panel g = c0 + q, q = t (c1 + t (c2 + ...))
-// of degree 7, where q is at most 2^-5 of c0 and each further term another 2^-5.5: c0 is a double,
+// of degree 7, where q is at most 2^-5 of g's size nearby and each further term another 2^-5.5: c0 is a double,
 // c1 .. c5 are pairs of floats evaluated with error-free products and sums (48 bits, so q carries
-// less than an ulp of g), c6 and c7 floats.  Both functions run in the two halves of the packed FP32
+// less than an ulp of that size; where g1 crosses zero its error is one of its size nearby, as a series
+// in FP64 has it), c6 and c7 floats.  Both functions run in the two halves of the packed FP32
 // instructions.  The pair becomes a double by integer operations (join), so FP64 is left with one
 // addition per function.  1024 FP64 runs of N = 128, 200 steps: 321 -> 109 ms (two additions), and
 // 98 -> 86 ms by the join.  Against 22-digit references (alpha 0.3 to 30) g1 is 2.1e-16 rms off, g2
