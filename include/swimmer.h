@@ -109,7 +109,9 @@ typedef struct swimmer_handle swimmer_handle;
 
 /* Create a handle on the current CUDA device: allocates the per-sample kernel tables,
  * the work queues and the TMCMC workspace for b_max samples (device memory owned by the
- * handle).  Synchronous.  *out receives the handle. */
+ * handle: per sample a kernel table, 86 KB in SWIMMER_FP64 or 37 KB in SWIMMER_FP32C, and less than
+ * 1 KB + 8 n_max bytes beside it; once, the table build's scratch, 123 KB times min(b_max, 4096)).
+ * Synchronous.  *out receives the handle. */
 int swimmer_init(const swimmer_config *cfg, swimmer_handle **out);
 
 /* Free everything the handle owns.  Synchronizes the device first. */

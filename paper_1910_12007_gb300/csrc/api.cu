@@ -158,7 +158,7 @@ extern "C" int swimmer_init(const swimmer_config *cfg, swimmer_handle **out) {
     const int B = cfg->b_max;
     ALLOC(h->tab64, (size_t)(cfg->precision == SWIMMER_FP64 ? B : 1) * TAB64_STRIDE);
     ALLOC(h->k1_scratch, (size_t)std::min(B, K1_SLICE) * K1_SCRATCH);
-    ALLOC(h->tab32, (size_t)B * TAB32_STRIDE);
+    ALLOC(h->tab32, (size_t)(cfg->precision == SWIMMER_FP64 ? 1 : B) * TAB32_STRIDE);
     if (cfg->precision != SWIMMER_FP64) ALLOC(h->pq, (size_t)B * cfg->n_max);
     ALLOC(h->sp, B);
     ALLOC(h->order, B);

@@ -112,7 +112,7 @@ struct swimmer_handle {
     // per-sample workspace (b_max samples)
     float4 *tab64;          // [b_max][TAB64_STRIDE] (FP32 handles: one, for kernel_eval and flow)
     double *k1_scratch;     // [min(b_max, K1_SLICE)][K1_SCRATCH] node values of the table build
-    float4 *tab32;          // [b_max][TAB32_STRIDE]
+    float4 *tab32;          // [b_max][TAB32_STRIDE] (FP64 handles: one, for kernel_eval)
     float2 *pq;             // FP32 handles: [b_max][n_max] preferred-curvature coefficients
     SampleParams *sp;       // [b_max]
     int *order;             // [b_max] processing order (longest first)
