@@ -175,7 +175,7 @@ __host__ __device__ inline bool symmetric_pays(int n) {
 
 // MODEL 0: the flagellum; 1: the full sperm model (head points and neck); 2: two sperm models
 // coupled by the fluid.  MAXT 1024, for runs above 512 points, is held to 64 registers and spills (360 to 560
-// bytes of loads a thread): 100 runs take, us a step, N = 600 2000, N = 768 4530, N = 1024 7400, a fifth to a
+// bytes of loads a thread): 100 runs take, us a step, N = 600 2000, N = 768 3120, N = 1024 7400, a fifth to a
 // quarter of what the Clenshaw kernel took (10500, 16700, 29100).  C CTAs (a cluster when C > 1) share a run.
 template <int MODEL, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) forward64_kernel(FwdArgs a, int C, int pw) {
@@ -705,11 +705,13 @@ size_t forward64_smem(int n_max, int panels, int threads, int pair_warps) {
 }
 
 // Warps of the symmetric pair sum in a launch with one run per CTA: at most one per unit, and 16, 8 or 4
-// as their arrays fit; 0 where it does not pay for the largest sample.
+// as their arrays fit; 0 where it does not pay for the largest sample, or, above 512 points, where a run is
+// alone on its SM, if fewer than 8 fit (100 runs, us a step: N = 768 8 warps 3120, every ordered pair in 32
+// 4530; N = 1024 4 warps 8010, 7400).
 int forward64_pair_warps(const swimmer_handle *h, int threads) {
-    const int n = h->cfg.n_max, nb = (n + 31) / 32;
+    const int n = h->cfg.n_max, nb = (n + 31) / 32, least = std::min(n > 512 ? 8 : 4, nb * nb);
     if (!symmetric_pays(n)) return 0;
-    for (int w = std::min(16, std::min(threads / 32, nb * nb)); w >= std::min(4, nb * nb); w >>= 1)
+    for (int w = std::min(16, std::min(threads / 32, nb * nb)); w >= least; w >>= 1)
         if (forward64_smem(n, handle_octaves(h) * F64_FINE, threads, w) + 2048 <= (size_t)h->max_smem) return w;
     return 0;
 }
