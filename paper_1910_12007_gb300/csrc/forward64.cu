@@ -14,7 +14,7 @@
 //     its next displacement.  In units of delta their last place was up to 1.5 times coarser and the errors
 //     of all steps added up: against extended precision (400 steps, N = 64) positions were 1.4e-16 to
 //     2.9e-16 off in the mean square, now below 0.72e-16, and the forces at the end 1.7 to 6 times as far as
-//     now.  It costs a lone run 2 % of its time (N = 64, 2000 steps 13.9 -> 14.2 ms), a batch 0.3 %;
+//     now.  It costs a lone run 1 % of its time (N = 64, 2000 steps 13.9 -> 14.05 ms), a batch 0.3 %;
 //   - (cos, sin)(omega t) is made for 32 steps at a time, a lane each, and the preferred curvature
 //     is P_k cos + Q_k sin; springs and curvature take one reciprocal square root each.
 // Of a run that has a CTA to itself every unordered pair is evaluated once, in the blocks and units of
@@ -25,7 +25,7 @@
 // smooth filament they read the same table panel).  A lone run is spread over a cluster of up to 16 SMs: a CTA owns
 // n / C points; forces and new positions go to every CTA's shared memory (double-buffered
 // positions, two cluster barriers a step).
-// Measured (whole calls): a lone run of N = 64, 2000 steps 53.1 -> 14.2 ms (26.5 -> 7.1 us a step) on a
+// Measured (whole calls): a lone run of N = 64, 2000 steps 53.1 -> 14.05 ms (26.5 -> 7.0 us a step) on a
 // cluster of 16; 1024 runs of N = 128, 200 steps 109 -> 65 ms (99 as a kernel of its own, 86 with 13
 // FP64 instructions a pair, 65 with the symmetric sum); 152 pairs of sperm models (148 points), 400
 // steps 44 -> 31.6 ms.
@@ -59,15 +59,16 @@ __device__ __forceinline__ double spring(double2 xi, double2 xj, const Rest &r, 
     return r.k2 * strain * rs;
 }
 
-// a value at the same place of every CTA of the cluster (its own among them: no branch in the loop;
-// C is even)
+// a value at the same place of every CTA of the cluster (its own among them: no branch in the loop).  One
+// thread sends them, a step's barrier waits for it: a lone run of N = 64 takes 14.20 ms with the loop unrolled by
+// 2, 14.05 by 4, 13.90 by 8, and 30 runs of N = 100 on clusters of 4 4.89, 4.89 and 4.93
 __device__ __forceinline__ void put_all(double2 *p, double2 v, int C) {
     if (C == 1) {
         *p = v;
         return;
     }
     const unsigned at = smem_addr(p);
-#pragma unroll 2
+#pragma unroll 4
     for (int r = 0; r < C; ++r)
         asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(remote(at, r)), "d"(v.x), "d"(v.y) : "memory");
 }
@@ -78,7 +79,7 @@ __device__ __forceinline__ void put_all(double2 *p, double2 v, double2 *q, doubl
         return;
     }
     const unsigned at = smem_addr(p), off = smem_addr(q) - at;
-#pragma unroll 2
+#pragma unroll 4
     for (int r = 0; r < C; ++r) {
         const unsigned to = remote(at, r);
         asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(to), "d"(v.x), "d"(v.y) : "memory");
